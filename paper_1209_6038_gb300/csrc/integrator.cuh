@@ -15,7 +15,7 @@
 //
 // Each lane owns one queued ray and refills from the queue when it finishes.  Every loop iteration
 // runs ONE uniform step evaluation for all lanes; the surface-crossing search (bisection prefix,
-// then Illinois regula falsi, see crossing() in physics.cuh) reuses that slot with a trial size.
+// then Illinois regula falsi, or Newton steps: Lane below) reuses that slot with a trial size.
 #pragma once
 
 #include "dfloat.cuh"
@@ -23,53 +23,35 @@
 
 namespace ck {
 
-// ------------------------------------------------------------------ FP64 stepper
-template <int VAR, int MODE, int INTEG>
-struct Stepper64 {
+// ------------------------------------------------------------------ FP64 steppers
+// What the FP64 steppers share: state, trial end point, event functions, metal mirror.
+template <int INTEG>
+struct State64 {
     typedef double real;
-    double y[6], k1[6], y1[6], e6[6], k7[6];
+    static constexpr bool FP64 = true;
+    double y[6], y1[6], e6[6];
     bool need_k1;
     int vm;  // 2 * variant + mode when VAR = MODE = V_ANY
 
-    // state of queue slot k; the first stage comes with it when the entry kernel computed it (Fermat form)
-    template <typename Q>
-    __device__ __forceinline__ void load(const Q &q, int k) {
-        y[0] = q.x[k]; y[1] = q.y[k]; y[2] = q.z[k];
-        y[3] = q.vx[k]; y[4] = q.vy[k]; y[5] = q.vz[k];
-        const double a0 = q.ax[k];
-        need_k1 = a0 != a0;
-        if (!need_k1) {
-            k1[0] = y[3]; k1[1] = y[4]; k1[2] = y[5];
-            k1[3] = a0; k1[4] = q.ay[k]; k1[5] = q.az[k];
-        }
-    }
-    __device__ __forceinline__ void eval(const Params &p, double s) {
-        if (INTEG == I_RK4) {
-            rk4_step<VAR, MODE>(p, y, s, y1, vm);
-        } else {
-            if (need_k1) rhs<VAR, MODE>(p, y, k1, vm);
-            need_k1 = false;
-            dp45_step<VAR, MODE>(p, y, k1, s, y1, e6, k7, vm);
-        }
-    }
     // DP5(4) step control (physics.cuh: dp_control); fac is the next-step factor
     __device__ __forceinline__ bool control(double tol, double &fac) const { return dp_control(y, y1, e6, tol, fac); }
     __device__ __forceinline__ double chord(const Params &p) const { return metal_chord(y[0], y[1], y1[0], y1[1], p.R1sq); }
     __device__ __forceinline__ double g_start(const Params &p, int ev) const { return event_g(p, ev, y); }
     __device__ __forceinline__ double g_end(const Params &p, int ev) const { return event_g(p, ev, y1); }
-    // d/ds of the event function at the end of the last trial step of size s, with the end point's
-    // derivative taken as the flow's, f(y1) = k7 (position part): the Newton slope of the crossing search
-    __device__ __forceinline__ double g_rate(int ev) const { return event_dg(ev, y1, k7); }
-    // the same at the start of the step, from k1 = f(y)
-    __device__ __forceinline__ double g_rate_start(int ev) const { return event_dg(ev, y, k1); }
-    __device__ __forceinline__ void take_step() {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) y[i] = y1[i];
-        if (INTEG == I_DP45) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i) k1[i] = k7[i];  // first stage of the next step (FSAL)
-        }
+    // surfaces behind the end point: bit ev is set iff event_g(ev, y1) > 0, decided by integer comparisons
+    __device__ __forceinline__ unsigned int crossed(const Params &p, int nev) const {
+        const double rr = fma(y1[0], y1[0], y1[1] * y1[1]), az = s64_abs(y1[2]);
+        unsigned int m = 0;
+        if (s64_gt_pos(rr, p.R2sq) && !s64_isnan(rr)) m |= 1u << EV_LAT;
+        if (s64_gt_pos(az, p.halfH) && !s64_isnan(az)) m |= __double2hiint(y1[2]) < 0 ? 1u << EV_BOT : 1u << EV_TOP;
+        if (nev == 4 && s64_gt_pos(p.R1sq, rr)) m |= 1u << EV_METAL;
+        return m;
     }
+    // d/ds of the event function at the end of the last trial step of size s, with the end point's
+    // derivative taken as the flow's, f(y1) (position part): the Newton slope of the crossing search
+    __device__ __forceinline__ double g_rate(int ev) const { return event_dg(ev, y1, y1 + 3); }
+    // the same at the start of the step, from f(y)
+    __device__ __forceinline__ double g_rate_start(int ev) const { return event_dg(ev, y, y + 3); }
     __device__ __forceinline__ void take_crossing() {
 #pragma unroll
         for (int i = 0; i < 6; ++i) y[i] = y1[i];
@@ -82,15 +64,108 @@ struct Stepper64 {
         y[4] -= 2.0 * vn * nm1;
         need_k1 = true;
     }
-    __device__ __forceinline__ void state(double out[6]) const {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) out[i] = y[i];
-    }
     // final state into queue slot k (FP64 format)
     template <typename Q>
     __device__ __forceinline__ void store(const Q &q, int k) const {
         q.x[k] = y[0]; q.y[k] = y[1]; q.z[k] = y[2];
         q.vx[k] = y[3]; q.vy[k] = y[4]; q.vz[k] = y[5];
+    }
+};
+
+// Fermat form: the compact steps, stages in shared memory (bind)
+template <int VAR, int MODE, int INTEG>
+struct Stepper64 : State64<INTEG> {
+    using B = State64<INTEG>;
+    using B::need_k1;
+    using B::vm;
+    using B::y;
+    using B::y1;
+    using B::e6;
+    static constexpr int SMEM_PER_THREAD = INTEG == I_DP45 ? DP_SLOTS * (int)sizeof(double) : 0;
+    double *kb;
+    int ks;
+    __device__ __forceinline__ void bind(double *smem) {
+        kb = smem + threadIdx.x;
+        ks = blockDim.x;
+    }
+    // state of queue slot k; the first stage comes with it when the entry kernel computed it
+    template <typename Q>
+    __device__ __forceinline__ void load(const Q &q, int k) {
+        y[0] = q.x[k]; y[1] = q.y[k]; y[2] = q.z[k];
+        y[3] = q.vx[k]; y[4] = q.vy[k]; y[5] = q.vz[k];
+        const double a0 = q.ax[k];
+        need_k1 = s64_isnan(a0);
+        if (INTEG == I_DP45 && !need_k1) {
+            kb[0] = y[3]; kb[ks] = y[4]; kb[2 * ks] = y[5];
+            kb[3 * ks] = a0; kb[4 * ks] = q.ay[k]; kb[5 * ks] = q.az[k];
+        }
+    }
+    template <int V, int M>
+    __device__ __forceinline__ void eval_medium(const Params &p, double s, bool first) {
+        if (INTEG == I_RK4) rk4_fermat<V, M>(p, y, s, y1);
+        else dp45_fermat<V, M>(p, y, s, first, kb, ks, y1, e6);
+    }
+    // lanes: the lanes of the warp that evaluate with this one
+    __device__ __forceinline__ void eval(const Params &p, double s, unsigned int lanes) {
+        const bool first = INTEG == I_DP45 && __any_sync(lanes, need_k1);
+        if (VAR != V_ANY) {
+            eval_medium<VAR, MODE>(p, s, first);
+        } else {
+            switch (vm) {
+            case 0: eval_medium<V_RADIAL, M_ORD>(p, s, first); break;
+            case 1: eval_medium<V_RADIAL, M_EXT>(p, s, first); break;
+            case 2: eval_medium<V_AZIMUTHAL, M_ORD>(p, s, first); break;
+            default: eval_medium<V_AZIMUTHAL, M_EXT>(p, s, first); break;
+            }
+        }
+        need_k1 = false;
+    }
+    __device__ __forceinline__ void take_step() {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) y[i] = y1[i];
+        if (INTEG == I_DP45) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) kb[i * ks] = kb[(36 + i) * ks];  // first stage of the next step (FSAL)
+        }
+    }
+};
+
+// Hamiltonian form: state (x, k), stages in registers
+template <int VAR, int MODE, int INTEG>
+struct StepperHam : State64<INTEG> {
+    using B = State64<INTEG>;
+    using B::need_k1;
+    using B::vm;
+    using B::y;
+    using B::y1;
+    using B::e6;
+    static constexpr int SMEM_PER_THREAD = 0;
+    double k1[6], k7[6];
+    __device__ __forceinline__ void bind(double *) {}
+    template <typename Q>
+    __device__ __forceinline__ void load(const Q &q, int k) {
+        y[0] = q.x[k]; y[1] = q.y[k]; y[2] = q.z[k];
+        y[3] = q.vx[k]; y[4] = q.vy[k]; y[5] = q.vz[k];
+        need_k1 = true;
+    }
+    __device__ __forceinline__ void eval(const Params &p, double s, unsigned int) {
+        if (INTEG == I_RK4) {
+            rk4_step<VAR, MODE, true>(p, y, s, y1, vm);
+        } else {
+            if (need_k1) rhs_ham<VAR, MODE>(p, y, k1, vm);
+            need_k1 = false;
+            dp45_step<VAR, MODE, true>(p, y, k1, s, y1, e6, k7, vm);
+        }
+    }
+    __device__ __forceinline__ double g_rate(int ev) const { return event_dg(ev, y1, k7); }
+    __device__ __forceinline__ double g_rate_start(int ev) const { return event_dg(ev, y, k1); }
+    __device__ __forceinline__ void take_step() {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) y[i] = y1[i];
+        if (INTEG == I_DP45) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) k1[i] = k7[i];  // first stage of the next step (FSAL)
+        }
     }
 };
 
@@ -272,11 +347,11 @@ template <int VAR, int MODE, int INTEG>
 __device__ __noinline__ void band_step_f64(const Params &p, const double *y, double s, double *yo, double *e,
                                            double *k7, int vm) {
     if (INTEG == I_RK4) {
-        rk4_step<VAR, MODE>(p, y, s, yo, vm);
+        rk4_step<VAR, MODE, false>(p, y, s, yo, vm);
     } else {
         double k1[6];
-        rhs<VAR, MODE>(p, y, k1, vm);
-        dp45_step<VAR, MODE>(p, y, k1, s, yo, e, k7, vm);
+        rhs_inline<VAR, MODE, false>(p, y, k1, vm);
+        dp45_step<VAR, MODE, false>(p, y, k1, s, yo, e, k7, vm);
     }
 }
 template <int VAR, int MODE>
@@ -311,12 +386,15 @@ __device__ __noinline__ void band_step_df(float R1h, float R1l, const df *y, flo
 template <int VAR, int MODE, int INTEG>
 struct StepperMixed {
     typedef float real;
+    static constexpr bool FP64 = false;
+    static constexpr int SMEM_PER_THREAD = 0;
     float yh[6], yl[6], k1[6];  // state (float-float) and first stage
     float y1h[6], y1l[6], e6[6], k7[6];
     float n6[6];  // rounding bound of the FP32 error estimate (noise floor)
     bool need_k1;
     int vm;  // 2 * variant + mode when VAR = MODE = V_ANY
 
+    __device__ __forceinline__ void bind(double *) {}
     // the queue holds the mixed path's states as float-float pairs: no conversion
     template <typename Q>
     __device__ __forceinline__ void load(const Q &q, int k) {
@@ -349,7 +427,7 @@ struct StepperMixed {
 #pragma unroll
         for (int i = 2; i < 6; ++i) t[i] = yh[i] + (yl[i] + d[i]);
     }
-    __device__ __forceinline__ void eval(const Params &p, float s) {
+    __device__ __forceinline__ void eval(const Params &p, float s, unsigned int) {
         if (p.band_df && island(p)) {  // double-float step from the float-float state
             df y[6], yo[6], e[6], kk7[6];
 #pragma unroll
@@ -505,6 +583,14 @@ struct StepperMixed {
     }
     __device__ __forceinline__ float g_start(const Params &p, int ev) const { return gval(p, ev, yh, yl); }
     __device__ __forceinline__ float g_end(const Params &p, int ev) const { return gval(p, ev, y1h, y1l); }
+    __device__ __forceinline__ unsigned int crossed(const Params &p, int nev) const {
+        unsigned int m = 0;
+        for (int e = 0; e < nev; ++e)
+            if (g_end(p, e) > 0.f) m |= 1u << e;
+        return m;
+    }
+    __device__ __forceinline__ float g_rate(int) const { return 1.f; }  // the search takes no Newton steps
+    __device__ __forceinline__ float g_rate_start(int) const { return 0.f; }
     __device__ __forceinline__ void take_step() {
 #pragma unroll
         for (int i = 0; i < 6; ++i) { yh[i] = y1h[i]; yl[i] = y1l[i]; }
@@ -538,8 +624,216 @@ struct StepperMixed {
     }
 };
 
-// ------------------------------------------------------------------ lane phases of the persistent loop
-// (k_wf_integrate in wavefront.cuh)
+// ------------------------------------------------------------------ one lane's ray: steps, crossings, mirror
 enum { PH_STEP = 0, PH_CROSS = 1, PH_FINAL = 2, PH_IDLE = 3 };
+
+// Comparisons of step sizes and event values: on the integer pipes for FP64 (each FP64 comparison would take a
+// slot of the FP64 unit for the whole warp).  a may be any value, lo and hi are not negative.
+__device__ __forceinline__ bool inside(double a, double lo, double hi) {
+    return __double_as_longlong(a) > __double_as_longlong(lo) && __double_as_longlong(a) < __double_as_longlong(hi);
+}
+__device__ __forceinline__ bool inside(float a, float lo, float hi) { return a > lo && a < hi; }
+__device__ __forceinline__ bool positive(double a) { return s64_positive(a); }
+__device__ __forceinline__ bool positive(float a) { return a > 0.f; }
+__device__ __forceinline__ bool le_pos(double a, double b) { return s64_le_pos(a, b); }  // 0 <= a or NaN, 0 <= b
+__device__ __forceinline__ bool le_pos(float a, float b) { return a <= b; }
+__device__ __forceinline__ double mag(double a) { return s64_abs(a); }
+__device__ __forceinline__ float mag(float a) { return fabsf(a); }
+
+// The ray of one lane: adaptive steps, the search for the surface that a step crosses, the metal mirror.  One
+// call of advance evaluates the stepper once, for stepping and searching lanes alike.
+// NEWTON: FP64 DP5(4) renders: when the ray moves towards the surface at both ends of the crossing step (one
+// crossing inside it), the search takes safeguarded Newton steps on the step function itself, the slope from the
+// end point's derivative f(y1), starting from a Newton step off the coarse step's end; otherwise, and for the
+// other paths, a bisection prefix and Illinois regula falsi.
+// EXACT: the regula falsi quotient as an IEEE division (the plain path) instead of a reciprocal product.
+template <typename S, int INTEG, bool NEWTON, bool EXACT>
+struct Lane {
+    typedef typename S::real R;
+    static constexpr double NEWTON_LAST = 1e-6;
+    static constexpr int prefix = bisect_prefix<INTEG>();
+    R h, t;
+    int steps, phase;
+    bool metal;
+    // crossing state
+    R hs, fac, lo, hi, glo, ghi, sbest, g1[4];
+    int ev, evbest, side, it;
+    bool newton, fin;
+    R snext;
+    unsigned int pending;
+
+    __device__ __forceinline__ void reset() {
+        phase = PH_IDLE;
+        h = t = hs = fac = lo = hi = glo = ghi = sbest = snext = (R)0;
+        steps = 0;
+        metal = newton = fin = false;
+        ev = side = it = 0;
+        evbest = -1;
+        pending = 0;
+    }
+    __device__ __forceinline__ void start(const Params &p) {
+        h = INTEG == I_RK4 ? (R)p.h_or_tol : (R)1e-3;
+        t = 0; steps = 0; metal = false;
+        phase = PH_STEP;
+    }
+    // One evaluation of st for the lanes `lanes` of the warp, which all call this together; mirrors: rays
+    // that reach the metal cylinder are mirrored (the others end there).  Returns the ray's status, -1 while
+    // it continues.
+    __device__ __forceinline__ int advance(const Params &p, S &st, unsigned int lanes, bool mirrors) {
+        const int nev = p.R1 > 0.0 ? 4 : 3;
+        const R tol = (R)p.h_or_tol;
+        const R conv = sizeof(R) == 8 ? (R)CROSS_REL_TOL : (R)2.4e-7;  // bracket resolution of the search
+        int status = -1;
+        if (phase == PH_STEP && (steps >= p.max_steps || (INTEG == I_DP45 && !le_pos((R)1e-14, h))))
+            status = CLOAK_RAY_STEP_LIMIT;
+        R s = phase == PH_STEP ? h : sbest;
+        if (phase == PH_CROSS) {
+            // next trial point: Newton (see above), or a bisection prefix, then Illinois regula falsi
+            if (newton) s = snext;
+            else if (it < prefix) s = (R)0.5 * (lo + hi);
+            else if (it - prefix < 60 && ghi > glo)
+                s = EXACT ? fma(lo, ghi, -(hi * glo)) / (ghi - glo) : fma(lo, ghi, -(hi * glo)) * rcp_nr(ghi - glo);
+            else s = (R)0.5 * (lo + hi);
+            if (!inside(s, lo, hi)) s = (R)0.5 * (lo + hi);
+        }
+        const unsigned int on = __ballot_sync(lanes, status < 0);
+        __syncwarp(lanes);  // a convergence point: keeps the compiler from splitting the evaluation by phase
+        if (status >= 0) return status;
+        st.eval(p, s, on);
+        bool land = false;
+        if (phase == PH_STEP) {
+            ++steps;
+            fac = 1;
+            bool accept = true;
+            if (INTEG == I_DP45) {
+                if (!st.control(tol, fac)) {
+                    h *= fmin(fac, (R)1);
+                    fac = 1;
+                    accept = false;
+                }
+            }
+            if (accept) {
+                pending = st.crossed(p, nev);
+                R sc = 0;
+                if (INTEG == I_DP45 && nev == 4 && !(pending & (1u << EV_METAL))) sc = st.chord(p);
+                if (positive(sc)) {
+                    h *= sc;  // retried: the step's chord passes through the metal cylinder
+                } else if (!pending) {
+                    st.take_step();
+                    t += h;
+                    h *= fac;
+                } else {
+                    #pragma unroll
+                    for (int e = 0; e < 4; ++e) g1[e] = st.g_end(p, e);
+                    hs = h;
+                    sbest = (R)1e30;
+                    evbest = -1;
+                    newton = false;
+                    fin = false;
+                    search(p, st);
+                    if (NEWTON) {
+                        const R d0 = (R)st.g_rate_start(ev), d1 = (R)st.g_rate(ev);
+                        if (d0 >= (R)0 && d1 > (R)0) {
+                            newton = true;
+                            R s0 = hs - ghi / d1;
+                            if (!(s0 > (R)0 && s0 < hs)) s0 = hs * (-glo / (ghi - glo));
+                            if (!(s0 > (R)0 && s0 < hs)) s0 = (R)0.5 * hs;
+                            snext = s0;
+                        }
+                    }
+                    phase = PH_CROSS;
+                }
+            }
+        } else if (phase == PH_CROSS) {
+            bool done = false;
+            const R gtol = (R)CROSS_G_TOL * (R)cross_g_scale(p, ev);
+            if (!inside(s, lo, hi)) {
+                done = true;
+            } else if (NEWTON && newton) {
+                // safeguarded Newton: keep the bracket, bisect when the step would leave it
+                const R gs = st.g_end(p, ev);
+                if (positive(gs)) { hi = s; ghi = gs; } else { lo = s; glo = gs; }
+                ++it;
+                if (fin || le_pos(mag(gs), gtol)) {
+                    // on the surface to rounding, or the trial point of a Newton correction below
+                    // NEWTON_LAST x the step: quadratic convergence put it within ~1e-12 of the step
+                    lo = s;
+                    hi = s;
+                    done = true;
+                } else {
+                    const R dg = (R)st.g_rate(ev);
+                    R sn = s - gs * rcp_nr(dg);
+                    if (!inside(sn, lo, hi)) sn = (R)0.5 * (lo + hi);
+                    else if (le_pos(mag(sn - s), (R)NEWTON_LAST * hs)) fin = true;
+                    snext = sn;
+                    if (hi - lo <= conv * hi || it >= 100) done = true;
+                }
+            } else {
+                R gs = st.g_end(p, ev);
+                if (it < prefix) {
+                    if (positive(gs)) { hi = s; ghi = gs; } else { lo = s; glo = gs; }
+                } else if (positive(gs)) {
+                    hi = s; ghi = gs;
+                    if (side == 1) glo *= (R)0.5;
+                    side = 1;
+                } else {
+                    lo = s; glo = gs;
+                    if (side == -1) ghi *= (R)0.5;
+                    side = -1;
+                }
+                ++it;
+                if (it >= prefix && hi - lo <= conv * hi) done = true;
+                // or a regula falsi trial point lies on the surface to rounding (Illinois approaches
+                // the root from one side, so the far end of the bracket may lag for many iterations)
+                if (!done && it > prefix && le_pos(mag(gs), gtol)) {
+                    lo = s;
+                    hi = s;
+                    done = true;
+                }
+                if (it >= prefix + 200) done = true;
+            }
+            if (done) {
+                R se = ev == EV_METAL ? lo : hi;
+                if (se < sbest) { sbest = se; evbest = ev; }
+                pending &= ~(1u << ev);
+                if (pending) {
+                    newton = false;  // the coarse step's end point is gone: bisection for further surfaces
+                    search(p, st);
+                } else if (S::FP64 && sbest == s && evbest == ev) {
+                    land = true;  // the last trial step ended on the crossing: no re-evaluation
+                } else {
+                    phase = PH_FINAL;
+                }
+            }
+        } else {
+            land = true;  // PH_FINAL: the evaluation landed on the crossing
+        }
+        if (land) {
+            st.take_crossing();
+            t += sbest;
+            h = hs * fac;
+            phase = PH_STEP;
+            if (evbest == EV_METAL) {
+                if (mirrors) {
+                    st.mirror();
+                    metal = true;
+                } else {
+                    status = CLOAK_RAY_SINGULAR;
+                }
+            } else {
+                status = metal ? CLOAK_RAY_HIT_METAL_EXITED : CLOAK_RAY_EXITED;
+            }
+        }
+        return status;
+    }
+    // start the search for the next pending surface
+    __device__ __forceinline__ void search(const Params &p, const S &st) {
+        ev = __ffs(pending) - 1;
+        lo = 0; hi = hs; glo = st.g_start(p, ev);
+        ghi = ev == 0 ? g1[0] : ev == 1 ? g1[1] : ev == 2 ? g1[2] : g1[3];
+        if (!(glo <= (R)0)) glo = 0;
+        side = 0; it = 0;
+    }
+};
 
 }  // namespace ck

@@ -220,6 +220,15 @@ __global__ void __launch_bounds__(128) k_refl_exit(Params p, Queue q2, float4 *r
     }
 }
 
+// FN<integrator, precision index>(arguments) for the handle's settings
+#define CK_INTEG_PREC(FN, ...)                                         \
+    const int prec = wf_prec(p);                                       \
+    if (p.integ == I_RK4)                                              \
+        return prec == 1   ? FN<I_RK4, 1>(__VA_ARGS__)                 \
+               : prec == 2 ? FN<I_RK4, 2>(__VA_ARGS__)                 \
+                           : FN<I_RK4, 0>(__VA_ARGS__);                \
+    return prec == 1 ? FN<I_DP45, 1>(__VA_ARGS__) : prec == 2 ? FN<I_DP45, 2>(__VA_ARGS__) : FN<I_DP45, 0>(__VA_ARGS__);
+
 template <int I, int PREC>
 static cudaError_t refl_ip(const Params &p, const Queue &q, const Queue &q2, float4 *refl, long long nrefl, int packet,
                            cudaStream_t st) {
@@ -233,22 +242,14 @@ static cudaError_t refl_ip(const Params &p, const Queue &q, const Queue &q2, flo
     k_wf_sort_scan<<<1, 32, 0, st>>>(q2, NBINS_BATCH, 0u);
     k_wf_sort_scatter<<<sms * 8, 256, 0, st>>>(q2);
     const int pk = packet > 0 ? packet : 128;
-    int nb = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, wf_integrate_kernel<V_ANY, V_ANY, I, PREC>(), pk, 0)) !=
-        cudaSuccess)
-        return e;
-    wf_integrate_kernel<V_ANY, V_ANY, I, PREC>()<<<(nb > 0 ? nb : 1) * sms, pk, 0, st>>>(p, q2);
+    if ((e = launch_wf_integrate<V_ANY, V_ANY, I, PREC>(p, q2, pk, sms, st)) != cudaSuccess) return e;
     k_refl_exit<<<sms * 16, 128, 0, st>>>(p, q2, refl);
     return cudaGetLastError();
 }
 
 cudaError_t launch_reflections(const Params &p, const Queue &q, const Queue &q2, float4 *refl, long long nrefl,
                                int packet, cudaStream_t st) {
-    if (p.integ == I_RK4)
-        return p.precision ? refl_ip<I_RK4, 1>(p, q, q2, refl, nrefl, packet, st)
-                           : refl_ip<I_RK4, 0>(p, q, q2, refl, nrefl, packet, st);
-    return p.precision ? refl_ip<I_DP45, 1>(p, q, q2, refl, nrefl, packet, st)
-                       : refl_ip<I_DP45, 0>(p, q, q2, refl, nrefl, packet, st);
+    CK_INTEG_PREC(refl_ip, p, q, q2, refl, nrefl, packet, st)
 }
 
 static inline void mark(cudaEvent_t *ev, int i, cudaStream_t st) {
@@ -274,12 +275,9 @@ static cudaError_t batch_ip(const Params &p, const ViewDev *views, int nviews, i
     k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS_BATCH, (unsigned int)(p.long_ray_blocks * pk * p.reserve_per_thread));
     k_wf_sort_scatter<<<sms * 8, 256, 0, st>>>(q);
     mark(ev, 1, st);
-    int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, wf_integrate_kernel<V_ANY, V_ANY, I, PREC>(), pk, 0);
-    if (e != cudaSuccess) return e;
     Params pl = p;
     pl.dedicated_blocks = p.long_ray_blocks;
-    wf_integrate_kernel<V_ANY, V_ANY, I, PREC>()<<<(nb > 0 ? nb : 1) * sms, pk, 0, st>>>(pl, q);
+    if ((e = launch_wf_integrate<V_ANY, V_ANY, I, PREC>(pl, q, pk, sms, st)) != cudaSuccess) return e;
     mark(ev, 2, st);
     k_batch_exit<<<sms * 16, 128, 0, st>>>(p, views, nviews, spp, seed, q, samples);
     mark(ev, 3, st);
@@ -352,33 +350,20 @@ static cudaError_t sur_data_ip(const Params &p, long long n, unsigned long long 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS_BATCH, 0u);
     k_wf_sort_scatter<<<sms * 8, 256, 0, st>>>(q);
-    int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, wf_integrate_kernel<V_ANY, V_ANY, I, PREC>(), 128, 0);
-    if (e != cudaSuccess) return e;
-    wf_integrate_kernel<V_ANY, V_ANY, I, PREC>()<<<(nb > 0 ? nb : 1) * sms, 128, 0, st>>>(p, q);
+    if ((e = launch_wf_integrate<V_ANY, V_ANY, I, PREC>(p, q, 128, sms, st)) != cudaSuccess) return e;
     k_sur_gen_exit<<<sms * 16, 128, 0, st>>>(p, seed, q, T_all);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sur_data(const Params &p, long long n, unsigned long long seed, const Queue &q, float *X_all,
                             float *T_all, cudaStream_t st) {
-    if (p.integ == I_RK4)
-        return p.precision ? sur_data_ip<I_RK4, 1>(p, n, seed, q, X_all, T_all, st)
-                           : sur_data_ip<I_RK4, 0>(p, n, seed, q, X_all, T_all, st);
-    return p.precision ? sur_data_ip<I_DP45, 1>(p, n, seed, q, X_all, T_all, st)
-                       : sur_data_ip<I_DP45, 0>(p, n, seed, q, X_all, T_all, st);
+    CK_INTEG_PREC(sur_data_ip, p, n, seed, q, X_all, T_all, st)
 }
 
 cudaError_t launch_batch(const Params &p, const ViewDev *views, int nviews, int spp, unsigned long long seed,
                          long long total, long long total_pix, const Queue &q, float4 *samples, int packet,
                          cudaStream_t st, cudaEvent_t *ev, const WfHook *hook) {
-    if (p.integ == I_RK4)
-        return p.precision
-                   ? batch_ip<I_RK4, 1>(p, views, nviews, spp, seed, total, total_pix, q, samples, packet, st, ev, hook)
-                   : batch_ip<I_RK4, 0>(p, views, nviews, spp, seed, total, total_pix, q, samples, packet, st, ev, hook);
-    return p.precision
-               ? batch_ip<I_DP45, 1>(p, views, nviews, spp, seed, total, total_pix, q, samples, packet, st, ev, hook)
-               : batch_ip<I_DP45, 0>(p, views, nviews, spp, seed, total, total_pix, q, samples, packet, st, ev, hook);
+    CK_INTEG_PREC(batch_ip, p, views, nviews, spp, seed, total, total_pix, q, samples, packet, st, ev, hook)
 }
 
 }  // namespace ck

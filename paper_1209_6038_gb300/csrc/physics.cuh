@@ -22,6 +22,7 @@
 #include <cstdint>
 
 #include "cloak.h"
+#include "soft64.cuh"
 
 namespace ck {
 
@@ -174,6 +175,83 @@ __device__ __forceinline__ void accel_fixed(T R1, T K, T invK, T x, T y, T vx, T
     ay = ar * cy + at * cx;
     az = azz;
 }
+// The same in double with every rounding written out, so that each copy of it in the library rounds alike:
+// M::mul is the product of two in-range factors, M::mulz one whose flagged factor may be exactly zero.
+struct MulHW {
+    static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+    static __device__ __forceinline__ double mulz(double a, double b, bool) { return __dmul_rn(a, b); }
+    static __device__ __forceinline__ double half(double a) { return __dmul_rn(0.5, a); }
+};
+struct MulInt {  // on the integer pipes (soft64.cuh)
+    static __device__ __forceinline__ double mul(double a, double b) { return s64_mul(a, b); }
+    static __device__ __forceinline__ double mulz(double a, double b, bool bzero) {
+        return s64_clear(bzero, s64_mul(a, s64_nonzero(bzero, b)));
+    }
+    static __device__ __forceinline__ double half(double a) { return s64_half(a); }
+};
+// Returns the range (s64_range) of what the products rest on: the inputs, and the sums that may cancel.
+template <typename M, int VAR, int MODE>
+__device__ __forceinline__ uint32_t accel64_form(double R1, double x, double y, double vx, double vy, double vz,
+                                                 double &ax, double &ay, double &az) {
+    const bool vz0 = s64_is_zero(vz);
+    const double r2 = fma(x, x, M::mul(y, y));
+    // 1 / r, as rsqrt_nr
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(r2));
+    const double e = fma(M::mul(-r2, y0), y0, 1.0);
+    const bool e0 = s64_is_zero(e);
+    const double ir = fma(M::mulz(y0, e, e0), fma(e, 0.375, 0.5), y0);
+    const double cx = M::mul(x, ir), cy = M::mul(y, ir);
+    const double vr = fma(vx, cx, M::mul(vy, cy));
+    const double vt = fma(vy, cx, -M::mul(vx, cy));
+    double r = 0.0, u;
+    if (VAR == V_RADIAL) {
+        r = M::mul(r2, ir);
+        u = r - R1;
+    } else {
+        u = fma(r2, ir, -R1);
+    }
+    const double g = M::mul(M::mul(2.0 * R1, ir), rcp_nr(u));  // f'/f
+    const double gvr = M::mul(-g, vr);
+    const double at = M::mul(gvr, vt);
+    double ar, br = 1.0;
+    if (MODE == M_EXT) {
+        const double R1ir2 = M::mul(M::mul(R1, ir), ir);
+        if (VAR == V_RADIAL) {
+            br = fma(M::mulz(u, vz, vz0), vz, -M::mul(M::mul(r, vt), vt));
+            ar = M::mul(M::mul(R1ir2, ir), br);
+            az = M::mulz(gvr, vz, vz0);
+        } else {
+            ar = M::mul(M::mul(-R1ir2, vt), vt);
+            az = 0.0;
+        }
+    } else {
+        br = fma(-vr, vr, fma(vz, vz, M::mul(vt, vt)));
+        ar = M::mul(M::half(g), br);
+        az = M::mulz(gvr, vz, vz0);
+    }
+    ax = fma(ar, cx, -M::mul(at, cy));
+    ay = fma(ar, cy, M::mul(at, cx));
+    uint32_t range = max(s64_range(x, y), s64_range(vx, vy));
+    range = max(range, max(s64_range(vr, vt), s64_range(u, R1)));
+    if (!vz0) range = max(range, s64_range(vz));
+    if (!e0) range = max(range, s64_range(e));
+    if (VAR == V_RADIAL || MODE == M_ORD) range = max(range, s64_range(br));
+    return range;
+}
+// Products on the integer pipes; a state out of their range (a component exactly zero, a point on r = R1)
+// takes the hardware's, with the same results.
+template <int VAR, int MODE>
+__device__ __forceinline__ void accel64(double R1, double x, double y, double vx, double vy, double vz, double &ax,
+                                        double &ay, double &az) {
+    if (VAR == V_TEST || (VAR == V_RADIAL && MODE == M_ORD)) {
+        ax = 0.0; ay = 0.0; az = 0.0;
+        return;
+    }
+    const uint32_t range = accel64_form<MulInt, VAR, MODE>(R1, x, y, vx, vy, vz, ax, ay, az);
+    if (!s64_ok(range)) accel64_form<MulHW, VAR, MODE>(R1, x, y, vx, vy, vz, ax, ay, az);
+}
+
 template <int VAR, int MODE, typename T>
 __device__ __forceinline__ void accel(T R1, T K, T invK, T x, T y, T vx, T vy, T vz, T &ax, T &ay, T &az, int vm) {
     if (VAR != V_ANY) {
@@ -238,38 +316,70 @@ __device__ __forceinline__ void ham_fixed(double R1, double K, double invK, cons
 }
 
 template <int VAR, int MODE>
+__device__ __forceinline__ void rhs_ham(const Params &p, const double y[6], double dy[6], int vm = 0) {
+    if (VAR != V_ANY) {
+        ham_fixed<VAR, MODE>(p.R1, p.K, p.invK, y, dy);
+        return;
+    }
+    switch (vm) {
+    case 0: ham_fixed<V_RADIAL, M_ORD>(p.R1, p.K, p.invK, y, dy); break;
+    case 1: ham_fixed<V_RADIAL, M_EXT>(p.R1, p.K, p.invK, y, dy); break;
+    case 2: ham_fixed<V_AZIMUTHAL, M_ORD>(p.R1, p.K, p.invK, y, dy); break;
+    default: ham_fixed<V_AZIMUTHAL, M_EXT>(p.R1, p.K, p.invK, y, dy); break;
+    }
+}
+
+template <int VAR, int MODE>
 __device__ __forceinline__ void rhs(const Params &p, const double y[6], double dy[6], int vm = 0) {
     if (p.formulation) {  // Hamiltonian form (radial and azimuthal cloaks)
-        if (VAR != V_ANY) {
-            ham_fixed<VAR, MODE>(p.R1, p.K, p.invK, y, dy);
-            return;
-        }
-        switch (vm) {
-        case 0: ham_fixed<V_RADIAL, M_ORD>(p.R1, p.K, p.invK, y, dy); break;
-        case 1: ham_fixed<V_RADIAL, M_EXT>(p.R1, p.K, p.invK, y, dy); break;
-        case 2: ham_fixed<V_AZIMUTHAL, M_ORD>(p.R1, p.K, p.invK, y, dy); break;
-        default: ham_fixed<V_AZIMUTHAL, M_EXT>(p.R1, p.K, p.invK, y, dy); break;
-        }
+        rhs_ham<VAR, MODE>(p, y, dy, vm);
         return;
     }
     dy[0] = y[3]; dy[1] = y[4]; dy[2] = y[5];
-    accel<VAR, MODE, double>(p.R1, p.K, p.invK, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], vm);
+    if (VAR != V_ANY) {
+        accel64<VAR, MODE>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]);
+        return;
+    }
+    switch (vm) {
+    case 0: accel64<V_RADIAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]); break;
+    case 1: accel64<V_RADIAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]); break;
+    case 2: accel64<V_AZIMUTHAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]); break;
+    default: accel64<V_AZIMUTHAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]); break;
+    }
 }
 
 // ------------------------------------------------------------------ integrators
-template <int VAR, int MODE>
+// Steps with the stages in registers: of the Hamiltonian form (HAM), or of the Fermat form with hardware products
+// (the mixed precision's band steps).
+template <int VAR, int MODE, bool HAM>
+__device__ __forceinline__ void rhs_inline(const Params &p, const double y[6], double dy[6], int vm) {
+    if (HAM) {
+        rhs_ham<VAR, MODE>(p, y, dy, vm);
+        return;
+    }
+    dy[0] = y[3]; dy[1] = y[4]; dy[2] = y[5];
+    dy[3] = dy[4] = dy[5] = 0.0;
+    const int m = VAR != V_ANY ? 2 * VAR + MODE : vm;
+    if (VAR != V_TEST && m == 1)
+        accel64_form<MulHW, V_RADIAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]);
+    else if (VAR != V_TEST && m == 2)
+        accel64_form<MulHW, V_AZIMUTHAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]);
+    else if (VAR != V_TEST && m == 3)
+        accel64_form<MulHW, V_AZIMUTHAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]);
+}
+template <int VAR, int MODE, bool HAM>
 __device__ __forceinline__ void rk4_step(const Params &p, const double y[6], double h, double out[6], int vm = 0) {
     double k[6], acc[6], t[6];
-    rhs<VAR, MODE>(p, y, k, vm);
+    rhs_inline<VAR, MODE, HAM>(p, y, k, vm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) { acc[i] = k[i]; t[i] = fma(0.5 * h, k[i], y[i]); }
-    rhs<VAR, MODE>(p, t, k, vm);
+    rhs_inline<VAR, MODE, HAM>(p, t, k, vm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) { acc[i] = fma(2.0, k[i], acc[i]); t[i] = fma(0.5 * h, k[i], y[i]); }
-    rhs<VAR, MODE>(p, t, k, vm);
+    rhs_inline<VAR, MODE, HAM>(p, t, k, vm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) { acc[i] = fma(2.0, k[i], acc[i]); t[i] = fma(h, k[i], y[i]); }
-    rhs<VAR, MODE>(p, t, k, vm);
+    rhs_inline<VAR, MODE, HAM>(p, t, k, vm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) out[i] = fma(h * (1.0 / 6.0), acc[i] + k[i], y[i]);
 }
@@ -292,7 +402,7 @@ struct DP {
 
 // Fifth-order solution of one DP step of size h from y with first stage k1 = f(y).
 // If err != nullptr also returns k7 = f(out) and the embedded error estimate.
-template <int VAR, int MODE>
+template <int VAR, int MODE, bool HAM>
 __device__ __forceinline__ void dp45_step(const Params &p, const double y[6], const double k1[6], double h,
                                           double out[6], double *err, double *k7, int vm = 0) {
     // stage points y + sum_l (h a_jl) k_l as FMA chains on the scaled coefficients (one FMA per term)
@@ -302,32 +412,32 @@ __device__ __forceinline__ void dp45_step(const Params &p, const double y[6], co
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = fma(c1, k1[i], y[i]);
     }
-    rhs<VAR, MODE>(p, t, k2, vm);
+    rhs_inline<VAR, MODE, HAM>(p, t, k2, vm);
     {
         const double c1 = h * DP::a31, c2 = h * DP::a32;
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = fma(c2, k2[i], fma(c1, k1[i], y[i]));
     }
-    rhs<VAR, MODE>(p, t, k3, vm);
+    rhs_inline<VAR, MODE, HAM>(p, t, k3, vm);
     {
         const double c1 = h * DP::a41, c2 = h * DP::a42, c3 = h * DP::a43;
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = fma(c3, k3[i], fma(c2, k2[i], fma(c1, k1[i], y[i])));
     }
-    rhs<VAR, MODE>(p, t, k4, vm);
+    rhs_inline<VAR, MODE, HAM>(p, t, k4, vm);
     {
         const double c1 = h * DP::a51, c2 = h * DP::a52, c3 = h * DP::a53, c4 = h * DP::a54;
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = fma(c4, k4[i], fma(c3, k3[i], fma(c2, k2[i], fma(c1, k1[i], y[i]))));
     }
-    rhs<VAR, MODE>(p, t, k5, vm);
+    rhs_inline<VAR, MODE, HAM>(p, t, k5, vm);
     {
         const double c1 = h * DP::a61, c2 = h * DP::a62, c3 = h * DP::a63, c4 = h * DP::a64, c5 = h * DP::a65;
 #pragma unroll
         for (int i = 0; i < 6; ++i)
             t[i] = fma(c5, k5[i], fma(c4, k4[i], fma(c3, k3[i], fma(c2, k2[i], fma(c1, k1[i], y[i])))));
     }
-    rhs<VAR, MODE>(p, t, k6, vm);
+    rhs_inline<VAR, MODE, HAM>(p, t, k6, vm);
     {
         const double c1 = h * DP::b1, c3 = h * DP::b3, c4 = h * DP::b4, c5 = h * DP::b5, c6 = h * DP::b6;
 #pragma unroll
@@ -335,7 +445,7 @@ __device__ __forceinline__ void dp45_step(const Params &p, const double y[6], co
             out[i] = fma(c6, k6[i], fma(c5, k5[i], fma(c4, k4[i], fma(c3, k3[i], fma(c1, k1[i], y[i])))));
     }
     if (err) {
-        rhs<VAR, MODE>(p, out, k7, vm);
+        rhs_inline<VAR, MODE, HAM>(p, out, k7, vm);
         const double c1 = h * DP::e1, c3 = h * DP::e3, c4 = h * DP::e4, c5 = h * DP::e5, c6 = h * DP::e6,
                      c7 = h * DP::e7;
 #pragma unroll
@@ -344,25 +454,152 @@ __device__ __forceinline__ void dp45_step(const Params &p, const double y[6], co
     }
 }
 
+// ------------------------------------------------------------------ the Fermat form's steps, compact
+// Bound by the FP64 unit (19 cycles per warp instruction and SM): with the products of the right-hand sides and
+// of the scaled tableau on the integer pipes (accel64, soft64.cuh), and comparisons and conversions of the step
+// control beside them, a radial extraordinary DP5(4) attempt takes some 235 FP64 instructions instead of 425.  The
+// right-hand side is one copy per medium, in a loop over the stages: it is some 700 instructions, and seven
+// inlined copies ran no faster than the FP64 unit alone because the warps waited for instructions.  The stages
+// live in shared memory (the loop indexes them), one column of DP_SLOTS doubles per thread, kb pointing at this
+// thread's first and ks threads per row; the roundings are those of dp45_step / rk4_step.  Twelve FP64 views of
+// 1920 x 1080 x 4: 1139 -> 746 ms; one such image 83 -> 53 ms; 30011 traced rays 15.8 -> 9.8 ms.
+constexpr int DP_SLOTS = 42;  // k1 .. k7, six components each
+// rows of the tableau for stages 2 .. 7 (the seventh is the fifth-order solution, without its zero b2), and
+// the error weights e1, e3 .. e6 in the order of the last row
+static __constant__ double c_dp_a[20] = {DP::a21, DP::a31, DP::a32, DP::a41, DP::a42, DP::a43, DP::a51,
+                                         DP::a52, DP::a53, DP::a54, DP::a61, DP::a62, DP::a63, DP::a64,
+                                         DP::a65, DP::b1,  DP::b3,  DP::b4,  DP::b5,  DP::b6};
+static __constant__ double c_dp_e[5] = {DP::e1, DP::e3, DP::e4, DP::e5, DP::e6};
+
+// Step of size h from y; k1 in slot 0, or evaluated here (first; uniform over the warp: evaluating the k1 that a
+// lane has already gives the same value).  y1: the fifth-order solution, e6: the error estimate,
+// slot 6: k7 = f(y1).  h: normal, far from the ends of the exponent range (h >= 1e-14 for a step; a trial
+// size of the crossing search is at least 2^-215 of one).
+template <int VAR, int MODE>
+__device__ __forceinline__ void dp45_fermat(const Params &p, const double y[6], double h, bool first, double *kb,
+                                            int ks, double y1[6], double e6[6]) {
+    if constexpr (VAR == V_TEST || (VAR == V_RADIAL && MODE == M_ORD)) {  // straight lines: every k is (v, 0)
+        const double b1 = h * DP::b1, b3 = h * DP::b3, b4 = h * DP::b4, b5 = h * DP::b5, b6 = h * DP::b6;
+        const double c1 = h * DP::e1, c3 = h * DP::e3, c4 = h * DP::e4, c5 = h * DP::e5, c6 = h * DP::e6,
+                     c7 = h * DP::e7;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const double v = y[3 + i];
+            y1[i] = fma(b6, v, fma(b5, v, fma(b4, v, fma(b3, v, fma(b1, v, y[i])))));
+            e6[i] = fma(c7, v, fma(c6, v, fma(c5, v, fma(c4, v, fma(c3, v, c1 * v)))));
+            y1[3 + i] = v;
+            e6[3 + i] = 0.0;
+        }
+    } else {
+        constexpr bool AZ = !(VAR == V_AZIMUTHAL && MODE == M_EXT);  // dv_z/dt is not identically zero
+        double t[6], a[3];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) e6[i] = 0.0;
+        int row = 0;
+#pragma unroll 1
+        for (int s = first ? 0 : 1; s < 7; ++s) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) t[i] = y[i];
+            const int terms = s < 6 ? s : 5;
+            const double *k = kb;
+#pragma unroll 1
+            for (int q = 0; q < terms; ++q) {
+                const double c = s64_mul(h, c_dp_a[row + q]);
+                const double k0 = k[0], k1 = k[ks], k3 = k[3 * ks], k4 = k[4 * ks];
+                t[0] = fma(c, k0, t[0]);
+                t[1] = fma(c, k1, t[1]);
+                t[3] = fma(c, k3, t[3]);
+                t[4] = fma(c, k4, t[4]);
+                double k5 = 0.0;
+                if (AZ) {
+                    k5 = k[5 * ks];
+                    t[5] = fma(c, k5, t[5]);
+                }
+                if (s == 6) {
+                    const double k2 = k[2 * ks], ce = s64_mul(h, c_dp_e[q]);
+                    t[2] = fma(c, k2, t[2]);
+                    e6[0] = fma(ce, k0, e6[0]);
+                    e6[1] = fma(ce, k1, e6[1]);
+                    e6[2] = fma(ce, k2, e6[2]);
+                    e6[3] = fma(ce, k3, e6[3]);
+                    e6[4] = fma(ce, k4, e6[4]);
+                    if (AZ) e6[5] = fma(ce, k5, e6[5]);
+                    if (q == 0) k += 6 * ks;  // no second stage in the solution
+                }
+                k += 6 * ks;
+            }
+            row += s;
+            accel64<VAR, MODE>(p.R1, t[0], t[1], t[3], t[4], t[5], a[0], a[1], a[2]);
+            double *ko = kb + 6 * s * ks;
+            ko[0] = t[3]; ko[ks] = t[4]; ko[2 * ks] = t[5];
+            ko[3 * ks] = a[0]; ko[4 * ks] = a[1]; ko[5 * ks] = a[2];
+        }
+        const double c7 = s64_mul(h, DP::e7);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) y1[i] = t[i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            e6[i] = fma(c7, t[3 + i], e6[i]);
+            if (i < 2 || AZ) e6[3 + i] = fma(c7, a[i], e6[3 + i]);
+        }
+    }
+}
+template <int VAR, int MODE>
+__device__ __forceinline__ void rk4_fermat(const Params &p, const double y[6], double h, double out[6]) {
+    if constexpr (VAR == V_TEST || (VAR == V_RADIAL && MODE == M_ORD)) {
+        const double h6 = h * (1.0 / 6.0);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const double v = y[3 + i];
+            out[i] = fma(h6, fma(2.0, v, fma(2.0, v, v)) + v, y[i]);
+            out[3 + i] = y[3 + i];
+        }
+    } else {
+        double acc[6], t[6], k[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) { acc[i] = 0.0; t[i] = y[i]; }
+        const double hh = 0.5 * h;
+#pragma unroll 1
+        for (int s = 0; s < 4; ++s) {
+            k[0] = t[3]; k[1] = t[4]; k[2] = t[5];
+            accel64<VAR, MODE>(p.R1, t[0], t[1], t[3], t[4], t[5], k[3], k[4], k[5]);
+            if (s == 3) break;
+            const double c = s < 2 ? hh : h, w = s == 0 ? 1.0 : 2.0;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                acc[i] = fma(w, k[i], acc[i]);
+                t[i] = fma(c, k[i], y[i]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 6; ++i) out[i] = fma(h * (1.0 / 6.0), acc[i] + k[i], y[i]);
+    }
+}
+
 // DP5(4) step control: accept iff |e_i| <= tol + tol max(|y_i|, |y1_i|) for every component
 // (decided in FP64); the step factor 0.9 err^(-1/5), clamped to [0.2, 5], is evaluated in FP32
 // (it only sets the next step size).  NaN -> reject with factor 0.2.
 __device__ __forceinline__ bool dp_control(const double y[6], const double y1[6], const double e6[6], double tol,
                                            double &fac) {
-    bool acc = true, bad = false;
+    bool acc = true, bad = false, ok = true;
     float fe = 0.f;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        double sc = tol + tol * fmax(fabs(y[i]), fabs(y1[i]));
-        double ae = fabs(e6[i]);
-        if (ae != ae) bad = true;
-        if (!(ae <= sc)) acc = false;
-        fe = fmaxf(fe, __fdividef((float)ae, (float)sc));
+    for (int i = 0; i < 6; ++i) {  // comparisons and conversions on the integer pipes
+        const double sc = fma(tol, fmax(s64_abs(y[i]), s64_abs(y1[i])), tol), ae = s64_abs(e6[i]);
+        if (s64_isnan(ae)) bad = true;
+        if (!s64_le_pos(ae, sc)) acc = false;
+        fe = fmaxf(fe, __fdividef(s64_to_float(ae, ok), s64_to_float(sc, ok)));
     }
     if (bad) { fac = 0.2; return false; }
+    if (!ok) {  // an error or scale beyond the float range
+        fe = 0.f;
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+            fe = fmaxf(fe, __fdividef((float)fabs(e6[i]), (float)fma(tol, fmax(fabs(y[i]), fabs(y1[i])), tol)));
+    }
     float f = fe == 0.f ? 5.f : fminf(5.f, fmaxf(0.2f, 0.9f * __powf(fe, -0.2f)));
     if (!(fe < 3.0e38f)) f = 0.2f;
-    fac = (double)f;
+    fac = s64_from_float(f);
     return acc;
 }
 
@@ -401,21 +638,13 @@ __device__ __forceinline__ double event_g(const Params &p, int ev, const double 
     }
 }
 
-// One step of size s from y with the integrator's own update (RK4, or the DP
-// fifth-order solution given k1 = f(y)).
-template <int VAR, int MODE, int INTEG>
-__device__ __forceinline__ void flow(const Params &p, const double y[6], const double k1[6], double s, double out[6],
-                                     int vm = 0) {
-    if (INTEG == I_RK4) rk4_step<VAR, MODE>(p, y, s, out, vm);
-    else dp45_step<VAR, MODE>(p, y, k1, s, out, nullptr, nullptr, vm);
-}
-
-// Root s* in (0, h] of g(flow_s(y)) for a surface crossed by the step (g(0) <= 0 < g(h)).
+// The crossing search (Lane, integrator.cuh): root s* in (0, h] of g(flow_s(y)) for a surface crossed by the step
+// (g(0) <= 0 < g(h)), flow_s the integrator's own update of size s.
 // When a coarse step crosses the surface more than once, the root is the one that
 // bisection of [0, h] converges to: the first halvings are plain bisection (same
 // midpoints as a pure bisection, so the same root is selected), then Illinois-modified
 // regula falsi finishes inside the remaining bracket.
-// Returns the end of the final bracket beyond the surface (exits) or before it (metal).
+// It ends at the end of the final bracket beyond the surface (exits) or before it (metal).
 // Halvings before regula falsi: 12 for fixed-step RK4 (coarse steps can cross a surface more than
 // once), 4 for the error-controlled DP5(4) steps.  Bracket resolution: 1e-13 of the step (FP64), or a
 // regula falsi point on the surface to rounding.
@@ -428,43 +657,6 @@ constexpr double CROSS_G_TOL = 4e-16;
 __device__ __forceinline__ double cross_g_scale(const Params &p, int ev) {
     return ev == EV_LAT ? p.R2sq : ev == EV_METAL ? p.R1sq : p.halfH;
 }
-template <int VAR, int MODE, int INTEG>
-__device__ double crossing(const Params &p, const double y[6], const double k1[6], double h, double ghi, int ev) {
-    double lo = 0.0, hi = h, glo = event_g(p, ev, y), t[6];
-    if (!(glo <= 0.0)) glo = 0.0;
-    for (int it = 0; it < bisect_prefix<INTEG>(); ++it) {
-        double mid = 0.5 * (lo + hi);
-        if (mid <= lo || mid >= hi) break;
-        flow<VAR, MODE, INTEG>(p, y, k1, mid, t);
-        double gm = event_g(p, ev, t);
-        if (gm > 0.0) { hi = mid; ghi = gm; }
-        else { lo = mid; glo = gm; }
-    }
-    int side = 0;
-    for (int it = 0; it < 200; ++it) {
-        if (hi - lo <= CROSS_REL_TOL * hi) break;
-        double s;
-        if (it < 60 && ghi > glo) s = (lo * ghi - hi * glo) / (ghi - glo);
-        else s = 0.5 * (lo + hi);
-        if (!(s > lo && s < hi)) s = 0.5 * (lo + hi);
-        if (!(s > lo && s < hi)) break;
-        flow<VAR, MODE, INTEG>(p, y, k1, s, t);
-        double gs = event_g(p, ev, t);
-        if (gs > 0.0) {
-            hi = s; ghi = gs;
-            if (side == 1) glo *= 0.5;
-            side = 1;
-        } else {
-            lo = s; glo = gs;
-            if (side == -1) ghi *= 0.5;
-            side = -1;
-        }
-        // the trial point lies on the surface to rounding: it is the crossing
-        if (fabs(gs) <= CROSS_G_TOL * cross_g_scale(p, ev)) return s;
-    }
-    return ev == EV_METAL ? lo : hi;
-}
-
 // First entry of o + s d into the finite cylinder r <= R2, |z| <= H/2.
 // face: EV_LAT / EV_TOP / EV_BOT, or -1 for a miss.
 __device__ __forceinline__ int cylinder_entry(const Params &p, const double o[3], const double d[3], double pt[3],

@@ -5,6 +5,9 @@
 // weights along the physical direction of light, and the room lookup.
 #pragma once
 
+#include <type_traits>
+
+#include "integrator.cuh"
 #include "physics.cuh"
 
 namespace ck {
@@ -125,87 +128,41 @@ __device__ __forceinline__ void leave(const Params &p, int ev, const double y[6]
     rec.tile_id = room_hit(p, x, dout, rgb);
 }
 
-// Whole ray, FP64.  rgb receives the room colour (0 when there is none).
-template <int VAR, int MODE, int INTEG>
-__device__ void trace_ray(const Params &p, const double o[3], const double d[3], cloak_record &rec, float rgb[3]) {
-    double y[6], k0[3], n_in[3], mat_in[5];
-    if (!enter<MODE>(p, o, d, rec, rgb, y, k0, n_in, mat_in)) return;
-    double t = 0.0, h = INTEG == I_RK4 ? p.h_or_tol : 1e-3, tol = p.h_or_tol;
-    int steps = 0;
-    bool metal = false, have_k1 = false;
-    const int nev = p.R1 > 0.0 ? 4 : 3;
-    double k1[6];
+// Whole ray, FP64 (HAM: Hamiltonian form), by the lanes of a warp together: `valid` lanes have a ray; smem: the
+// block's shared memory of the stepper.  rgb receives the room colour (0 when there is none).
+template <int VAR, int MODE, int INTEG, bool HAM>
+using PlainStepper = typename std::conditional<HAM, StepperHam<VAR, MODE, INTEG>, Stepper64<VAR, MODE, INTEG>>::type;
+template <int VAR, int MODE, int INTEG, bool HAM>
+__device__ __forceinline__ void trace_ray(const Params &p, bool valid, const double o[3], const double d[3], double *smem,
+                                          cloak_record &rec, float rgb[3]) {
+    typedef PlainStepper<VAR, MODE, INTEG, HAM> S;
+    S st;
+    st.vm = 2 * VAR + MODE;
+    st.bind(smem);
+    double k0[3], n_in[3], mat_in[5];
+    Lane<S, INTEG, false, true> ray;
+    ray.reset();
+    if (valid && enter<MODE>(p, o, d, rec, rgb, st.y, k0, n_in, mat_in)) ray.start(p);
+    st.need_k1 = true;
+    int status = -1;
     for (;;) {
-        if (steps >= p.max_steps || (INTEG == I_DP45 && h < 1e-14)) {
-            rec.status = CLOAK_RAY_STEP_LIMIT;
-            break;
-        }
-        double y1[6], fac = 1.0, k7[6];
-        if (INTEG == I_RK4) {
-            rk4_step<VAR, MODE>(p, y, h, y1);
-            ++steps;
-        } else {
-            if (!have_k1) { rhs<VAR, MODE>(p, y, k1); have_k1 = true; }
-            double e6[6];
-            dp45_step<VAR, MODE>(p, y, k1, h, y1, e6, k7);
-            ++steps;
-            if (!dp_control(y, y1, e6, tol, fac)) {
-                h *= fmin(fac, 1.0);
-                continue;
-            }
-        }
-        if (INTEG == I_DP45 && nev == 4 && event_g(p, EV_METAL, y1) <= 0.0) {
-            double sc = metal_chord(y[0], y[1], y1[0], y1[1], p.R1sq);
-            if (sc > 0.0) {
-                h *= sc;
-                continue;
-            }
-        }
-        int evh = -1;
-        double sh = 1e300;
-        for (int ev = 0; ev < nev; ++ev) {
-            double g1 = event_g(p, ev, y1);
-            if (g1 > 0.0) {
-                double s = crossing<VAR, MODE, INTEG>(p, y, k1, h, g1, ev);
-                if (s < sh) { sh = s; evh = ev; }
-            }
-        }
-        if (evh < 0) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i) y[i] = y1[i];
-            t += h;
-            h *= fac;
-            if (INTEG == I_DP45) {
-#pragma unroll
-                for (int i = 0; i < 6; ++i) k1[i] = k7[i];  // first stage of the next step (FSAL)
-            }
-            continue;
-        }
-        flow<VAR, MODE, INTEG>(p, y, k1, sh, y1);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) y[i] = y1[i];
-        t += sh;
-        h *= fac;
-        have_k1 = false;
-        if (evh == EV_METAL) {
-            if (VAR == V_RADIAL && MODE == M_ORD) {  // Sect. 4: single mirror ray, c-hat along the metal normal
-                double r = hypot(y[0], y[1]), nm0 = y[0] / r, nm1 = y[1] / r;
-                double vn = y[3] * nm0 + y[4] * nm1;
-                y[3] -= 2.0 * vn * nm0;
-                y[4] -= 2.0 * vn * nm1;
-                metal = true;
-                continue;
-            }
-            rec.status = CLOAK_RAY_SINGULAR;
-            break;
-        }
-        leave<MODE>(p, evh, y, d, k0, n_in, mat_in, metal, t, steps, rec, rgb);
+        const bool live = ray.phase != PH_IDLE;
+        const unsigned int lm = __ballot_sync(0xffffffffu, live);
+        if (!lm) break;
+        if (!live) continue;
+        status = ray.advance(p, st, lm, VAR == V_RADIAL && MODE == M_ORD);
+        if (status >= 0) ray.phase = PH_IDLE;
+    }
+    if (status < 0) return;  // never entered
+    if (status == CLOAK_RAY_EXITED || status == CLOAK_RAY_HIT_METAL_EXITED) {
+        leave<MODE>(p, ray.evbest, st.y, d, k0, n_in, mat_in, ray.metal, ray.t, ray.steps, rec, rgb);
         return;
     }
     // STEP_LIMIT or SINGULAR
-    rec.steps = steps;
-    rec.tof = t;
-    rec.exit_pos[0] = y[0]; rec.exit_pos[1] = y[1]; rec.exit_pos[2] = y[2];
+    rec.status = status;
+    rec.steps = ray.steps;
+    rec.tof = ray.t;
+    rec.exit_pos[0] = st.y[0]; rec.exit_pos[1] = st.y[1]; rec.exit_pos[2] = st.y[2];
     set_vec(rec.exit_dir, d);
 }
 

@@ -220,22 +220,19 @@ __global__ void __launch_bounds__(128) k_wf_entry(Params p, int spp, unsigned lo
 __global__ void k_wf_sort_scan(Queue q, int nbins, unsigned int reserve);
 __global__ void k_wf_sort_scatter(Queue q);
 
+// PREC: 0 FP64 (Fermat form), 1 mixed precision, 2 FP64 Hamiltonian form
+template <int VAR, int MODE, int INTEG, int PREC>
+using WfStepper = typename std::conditional<
+    PREC == 0, Stepper64<VAR, MODE, INTEG>,
+    typename std::conditional<PREC == 1, StepperMixed<VAR, MODE, INTEG>, StepperHam<VAR, MODE, INTEG>>::type>::type;
 template <int VAR, int MODE, int INTEG, int PREC>
 __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &q) {
-    typedef typename std::conditional<PREC == 0, Stepper64<VAR, MODE, INTEG>, StepperMixed<VAR, MODE, INTEG>>::type S;
-    typedef typename S::real R;
+    typedef WfStepper<VAR, MODE, INTEG, PREC> S;
+    extern __shared__ double wf_smem[];
     S st;
     st.vm = 0;
+    st.bind(wf_smem);
     const unsigned int n = q.count[2];  // rays left to integrate after the sort
-    const int nev = p.R1 > 0.0 ? 4 : 3;
-    const R tol = (R)p.h_or_tol, h0 = INTEG == I_RK4 ? (R)p.h_or_tol : (R)1e-3;
-    const R conv = sizeof(R) == 8 ? (R)CROSS_REL_TOL : (R)2.4e-7;  // bracket resolution of the crossing search
-    constexpr int prefix = bisect_prefix<INTEG>();
-    // FP64 DP5(4): when the ray moves towards the surface at both ends of the crossing step (one crossing
-    // inside it), the search takes safeguarded Newton steps on the step function itself, the slope from
-    // the end point's derivative f(y1), starting from a Newton step off the coarse step's end
-    constexpr bool NEWTON = INTEG == I_DP45 && PREC == 0;
-    constexpr double NEWTON_LAST = 1e-6;
     // medium segments of the permutation (batch: one per medium/mode; a lane draws rays from its
     // warp's current segment, so that the lanes of a warp evaluate one medium's equations)
     // the first segment is chosen per SM, so that the warps resident on one SM run one medium's code
@@ -266,16 +263,9 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
             if (__shfl_sync(0xffffffffu, f, 0)) return;  // the whole warp leaves
         }
     }
-    // lane state
-    R h = h0, t = 0;
-    int steps = 0, phase = PH_IDLE, slot = -1;
-    bool metal = false;
-    // crossing state
-    R hs = 0, fac = 1, lo = 0, hi = 0, glo = 0, ghi = 0, sbest = 0, g1[4];
-    int ev = 0, evbest = -1, side = 0, it = 0;
-    bool newton = false, fin = false;
-    R snext = 0;
-    unsigned int pending = 0;
+    Lane<S, INTEG, INTEG == I_DP45 && PREC != 1, false> ray;
+    ray.reset();
+    int slot = -1;
     bool drained = false;  // the queue had no ray left for this lane
 
     // Every lane of a warp stays in the loop until the whole warp is drained, and the warp reconverges
@@ -283,7 +273,8 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
     // (stepping and crossing search alike).
     for (;;) {
         // ---- refill: a lane without a ray takes the next queued one
-        if (phase == PH_IDLE && !drained) {
+        if (ray.phase == PH_IDLE && !drained) {
+            int phase = PH_IDLE;
             if (VAR == V_ANY) {
                 if (reserve) {  // a long-ray lane: the reserved rays first
                     const unsigned int k = atomicAdd(q.count + 10, 1u);
@@ -330,178 +321,30 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
             }
             if (phase == PH_STEP) {
                 st.load(q, slot);
-                h = h0; t = 0; steps = 0; metal = false;
+                ray.start(p);
             }
         }
-        const bool live = phase != PH_IDLE;
+        const bool live = ray.phase != PH_IDLE;
         if (!live) drained = true;
         const unsigned int lm = __ballot_sync(0xffffffffu, live);
         if (!lm) break;     // the whole warp is drained
         if (!live) continue;
-        int status = -1;
-        if (phase == PH_STEP && (steps >= p.max_steps || (INTEG == I_DP45 && h < (R)1e-14))) status = CLOAK_RAY_STEP_LIMIT;
-        R s = phase == PH_STEP ? h : sbest;
-        if (phase == PH_CROSS) {
-            // next trial point: Newton (see above), or a bisection prefix, then Illinois regula falsi
-            // (see crossing())
-            if (newton) s = snext;
-            else if (it < prefix) s = (R)0.5 * (lo + hi);
-            else if (it - prefix < 60 && ghi > glo) s = (lo * ghi - hi * glo) * rcp_nr(ghi - glo);
-            else s = (R)0.5 * (lo + hi);
-            if (!(s > lo && s < hi)) s = (R)0.5 * (lo + hi);
-        }
-        __syncwarp(lm);  // a convergence point: keeps the compiler from splitting the evaluation by phase
-        bool land = false;
-        if (status < 0) {
-            st.eval(p, s);
-            if (phase == PH_STEP) {
-                ++steps;
-                fac = 1;
-                bool accept = true;
-                if (INTEG == I_DP45) {
-                    if (!st.control(tol, fac)) {
-                        h *= fmin(fac, (R)1);
-                        fac = 1;
-                        accept = false;
-                    }
-                }
-                if (accept) {
-                    pending = 0;
-                    for (int e = 0; e < nev; ++e) {
-                        g1[e] = st.g_end(p, e);
-                        if (g1[e] > (R)0) pending |= 1u << e;
-                    }
-                    R sc = 0;
-                    if (INTEG == I_DP45 && nev == 4 && !(pending & (1u << EV_METAL))) sc = st.chord(p);
-                    if (sc > (R)0) {
-                        h *= sc;  // retried: the step's chord passes through the metal cylinder
-                    } else if (!pending) {
-                        st.take_step();
-                        t += h;
-                        h *= fac;
-                    } else {
-                        hs = h;
-                        sbest = (R)1e30;
-                        evbest = -1;
-                        ev = __ffs(pending) - 1;
-                        lo = 0; hi = hs; glo = st.g_start(p, ev); ghi = g1[ev];
-                        if (!(glo <= (R)0)) glo = 0;
-                        side = 0; it = 0;
-                        newton = false;
-                        fin = false;
-                        if constexpr (NEWTON) {
-                            const R d0 = (R)st.g_rate_start(ev), d1 = (R)st.g_rate(ev);
-                            if (d0 >= (R)0 && d1 > (R)0) {
-                                newton = true;
-                                R s0 = hs - ghi / d1;
-                                if (!(s0 > (R)0 && s0 < hs)) s0 = hs * (-glo / (ghi - glo));
-                                if (!(s0 > (R)0 && s0 < hs)) s0 = (R)0.5 * hs;
-                                snext = s0;
-                            }
-                        }
-                        phase = PH_CROSS;
-                    }
-                }
-            } else if (phase == PH_CROSS) {
-                bool done = false;
-                if (!(s > lo && s < hi)) {
-                    done = true;
-                } else if (NEWTON && newton) {
-                    // safeguarded Newton: keep the bracket, bisect when the step would leave it
-                    const R gs = st.g_end(p, ev);
-                    if (gs > (R)0) { hi = s; ghi = gs; } else { lo = s; glo = gs; }
-                    ++it;
-                    const R gtol = (R)CROSS_G_TOL * (R)cross_g_scale(p, ev);
-                    if (fin || fabs(gs) <= gtol) {
-                        // on the surface to rounding, or the trial point of a Newton correction below
-                        // NEWTON_LAST x the step: quadratic convergence put it within ~1e-12 of the step
-                        lo = s;
-                        hi = s;
-                        done = true;
-                    } else {
-                        R dg = (R)1;
-                        if constexpr (NEWTON) dg = (R)st.g_rate(ev);
-                        R sn = s - gs * rcp_nr(dg);
-                        if (!(sn > lo && sn < hi)) sn = (R)0.5 * (lo + hi);
-                        else if (fabs(sn - s) <= (R)NEWTON_LAST * hs) fin = true;
-                        snext = sn;
-                        if (hi - lo <= conv * hi || it >= 100) done = true;
-                    }
-                } else {
-                    R gs = st.g_end(p, ev);
-                    if (it < prefix) {
-                        if (gs > (R)0) { hi = s; ghi = gs; } else { lo = s; glo = gs; }
-                    } else if (gs > (R)0) {
-                        hi = s; ghi = gs;
-                        if (side == 1) glo *= (R)0.5;
-                        side = 1;
-                    } else {
-                        lo = s; glo = gs;
-                        if (side == -1) ghi *= (R)0.5;
-                        side = -1;
-                    }
-                    ++it;
-                    if (it >= prefix && hi - lo <= conv * hi) done = true;
-                    // or a regula falsi trial point lies on the surface to rounding (Illinois approaches
-                    // the root from one side, so the far end of the bracket may lag for many iterations)
-                    const R gtol = (R)CROSS_G_TOL * (R)cross_g_scale(p, ev);
-                    if (!done && it > prefix && fabs(gs) <= gtol) {
-                        lo = s;
-                        hi = s;
-                        done = true;
-                    }
-                    if (it >= prefix + 200) done = true;
-                }
-                if (done) {
-                    R se = ev == EV_METAL ? lo : hi;
-                    if (se < sbest) { sbest = se; evbest = ev; }
-                    pending &= ~(1u << ev);
-                    if (pending) {
-                        ev = __ffs(pending) - 1;
-                        lo = 0; hi = hs; glo = st.g_start(p, ev); ghi = g1[ev];
-                        if (!(glo <= (R)0)) glo = 0;
-                        side = 0; it = 0;
-                        newton = false;  // the coarse step's end point is gone: bisection for further surfaces
-                    } else if (PREC == 0 && sbest == s && evbest == ev) {
-                        land = true;  // the last trial step ended on the crossing: no re-evaluation
-                    } else {
-                        phase = PH_FINAL;
-                    }
-                }
-            } else {
-                land = true;  // PH_FINAL: the evaluation landed on the crossing
-            }
-            if (land) {
-                st.take_crossing();
-                t += sbest;
-                h = hs * fac;
-                phase = PH_STEP;
-                if (evbest == EV_METAL) {
-                    if ((VAR == V_RADIAL && MODE == M_ORD) || (VAR == V_ANY && st.vm == 0)) {
-                        st.mirror();
-                        metal = true;
-                    } else {
-                        status = CLOAK_RAY_SINGULAR;
-                    }
-                } else {
-                    status = metal ? CLOAK_RAY_HIT_METAL_EXITED : CLOAK_RAY_EXITED;
-                }
-            }
-        }
+        const bool mirrors = (VAR == V_RADIAL && MODE == M_ORD) || (VAR == V_ANY && st.vm == 0);
+        const int status = ray.advance(p, st, lm, mirrors);
         if (status >= 0) {  // ray finished: write back (in the queue's state format), lane becomes idle
             st.store(q, slot);
-            q.t[slot] = (double)t;
+            q.t[slot] = (double)ray.t;
             q.status[slot] = status;
-            q.steps[slot] = steps;
-            q.face[slot] = evbest;
-            phase = PH_IDLE;
+            q.steps[slot] = ray.steps;
+            q.face[slot] = ray.evbest;
+            ray.phase = PH_IDLE;
         }
     }
 }
 
-// The FP64 integrator keeps the compiler's register choice (148-151 registers, three blocks of 128
-// threads per SM); the mixed one is held to 128 registers for four blocks per SM -- its FP32 steps are
-// latency-bound and gain from the extra warps, while the rare band steps near R1 may spill.
+// The FP64 integrator keeps the compiler's register choice; the mixed one is held to 128 registers for four
+// blocks per SM -- its FP32 steps are latency-bound and gain from the extra warps, while the rare band steps
+// near R1 may spill.
 template <int VAR, int MODE, int INTEG, int PREC>
 __global__ void __launch_bounds__(128) k_wf_integrate(Params p, Queue q) {
     wf_integrate_body<VAR, MODE, INTEG, PREC>(p, q);
@@ -512,8 +355,21 @@ __global__ void __launch_bounds__(128, 4) k_wf_integrate_mixed(const __grid_cons
 }
 template <int VAR, int MODE, int INTEG, int PREC>
 constexpr auto wf_integrate_kernel() {
-    if constexpr (PREC == 0) return k_wf_integrate<VAR, MODE, INTEG, PREC>;
+    if constexpr (PREC != 1) return k_wf_integrate<VAR, MODE, INTEG, PREC>;
     else return k_wf_integrate_mixed<VAR, MODE, INTEG, PREC>;
+}
+// the kernel's precision index from the handle's settings
+inline int wf_prec(const Params &p) { return p.precision ? 1 : p.formulation ? 2 : 0; }
+// Launch the persistent integrator over the sorted queue: exactly the resident grid.
+template <int VAR, int MODE, int INTEG, int PREC>
+cudaError_t launch_wf_integrate(const Params &p, const Queue &q, int packet, int sms, cudaStream_t st) {
+    constexpr auto kern = wf_integrate_kernel<VAR, MODE, INTEG, PREC>();
+    const size_t smem = (size_t)WfStepper<VAR, MODE, INTEG, PREC>::SMEM_PER_THREAD * packet;
+    int nb = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, packet, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(nb > 0 ? nb : 1) * sms, packet, smem, st>>>(p, q);
+    return cudaGetLastError();
 }
 
 // Exit of queue slot k: refraction into vacuum at the crossed face, the Eq. 12 factor of the exit face
@@ -606,16 +462,9 @@ static cudaError_t wavefront_vmip(const Params &p, int spp, unsigned long long s
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[1], st);
-    // persistent integrator: exactly the resident grid
-    int nb = 0;
-    constexpr auto kern = wf_integrate_kernel<V, M, I, PREC>();
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, pk, 0);
-    if (e != cudaSuccess) return e;
     Params pl = p;
     pl.dedicated_blocks = p.long_ray_blocks;
-    kern<<<(nb > 0 ? nb : 1) * sms, pk, 0, st>>>(pl, q);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if ((e = launch_wf_integrate<V, M, I, PREC>(pl, q, pk, sms, st)) != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[2], st);
     k_wf_exit<V, M><<<sms * 16, 128, 0, st>>>(p, spp, seed, q, samples, recs);
     e = cudaGetLastError();
@@ -626,7 +475,11 @@ static cudaError_t wavefront_vmip(const Params &p, int spp, unsigned long long s
 template <int V, int M, int I>
 static cudaError_t wavefront_vmi(const Params &p, int spp, unsigned long long seed, const Queue &q, float4 *samples,
                                  cloak_record *recs, int packet, cudaStream_t st, cudaEvent_t *ev, const WfHook *hook) {
-    if (p.precision != 0) return wavefront_vmip<V, M, I, 1>(p, spp, seed, q, samples, recs, packet, st, ev, hook);
+    const int prec = wf_prec(p);
+    if (prec == 1) return wavefront_vmip<V, M, I, 1>(p, spp, seed, q, samples, recs, packet, st, ev, hook);
+    if constexpr (V != V_TEST) {
+        if (prec == 2) return wavefront_vmip<V, M, I, 2>(p, spp, seed, q, samples, recs, packet, st, ev, hook);
+    }
     return wavefront_vmip<V, M, I, 0>(p, spp, seed, q, samples, recs, packet, st, ev, hook);
 }
 
