@@ -35,18 +35,24 @@ struct State64 {
 
     // DP5(4) step control (physics.cuh: dp_control); fac is the next-step factor
     __device__ __forceinline__ bool control(double tol, double &fac) const { return dp_control(y, y1, e6, tol, fac); }
-    __device__ __forceinline__ double chord(const Params &p) const { return metal_chord(y[0], y[1], y1[0], y1[1], p.R1sq); }
+    __device__ __forceinline__ double chord(const Params &p) const {
+        if (!chord_near(s64_truncate(y[0]), s64_truncate(y[1]), s64_truncate(y1[0]), s64_truncate(y1[1]), p.R1f)) return 0.0;
+        return metal_chord(y[0], y[1], y1[0], y1[1], p.R1sq);
+    }
     __device__ __forceinline__ double g_start(const Params &p, int ev) const { return event_g(p, ev, y); }
     __device__ __forceinline__ double g_end(const Params &p, int ev) const { return event_g(p, ev, y1); }
+    double rr;  // r^2 at y1, where the step leaves it (DP5(4) of the Fermat form)
     // surfaces behind the end point: bit ev is set iff event_g(ev, y1) > 0, decided by integer comparisons
-    __device__ __forceinline__ unsigned int crossed(const Params &p, int nev) const {
-        const double rr = fma(y1[0], y1[0], y1[1] * y1[1]), az = s64_abs(y1[2]);
+    template <bool RR>
+    __device__ __forceinline__ unsigned int crossed_rr(const Params &p, int nev) const {
+        const double r2 = RR ? rr : fma(y1[0], y1[0], __dmul_rn(y1[1], y1[1])), az = s64_abs(y1[2]);
         unsigned int m = 0;
-        if (s64_gt_pos(rr, p.R2sq) && !s64_isnan(rr)) m |= 1u << EV_LAT;
+        if (s64_gt_pos(r2, p.R2sq) && !s64_isnan(r2)) m |= 1u << EV_LAT;
         if (s64_gt_pos(az, p.halfH) && !s64_isnan(az)) m |= __double2hiint(y1[2]) < 0 ? 1u << EV_BOT : 1u << EV_TOP;
-        if (nev == 4 && s64_gt_pos(p.R1sq, rr)) m |= 1u << EV_METAL;
+        if (nev == 4 && s64_gt_pos(p.R1sq, r2)) m |= 1u << EV_METAL;
         return m;
     }
+    __device__ __forceinline__ unsigned int crossed(const Params &p, int nev) const { return crossed_rr<false>(p, nev); }
     // d/ds of the event function at the end of the last trial step of size s, with the end point's
     // derivative taken as the flow's, f(y1) (position part): the Newton slope of the crossing search
     __device__ __forceinline__ double g_rate(int ev) const { return event_dg(ev, y1, y1 + 3); }
@@ -64,6 +70,8 @@ struct State64 {
         y[4] -= 2.0 * vn * nm1;
         need_k1 = true;
     }
+    // after a change of y from outside
+    __device__ __forceinline__ void begin() { need_k1 = true; }
     // final state into queue slot k (FP64 format)
     template <typename Q>
     __device__ __forceinline__ void store(const Q &q, int k) const {
@@ -81,6 +89,10 @@ struct Stepper64 : State64<INTEG> {
     using B::y;
     using B::y1;
     using B::e6;
+    using B::rr;
+    __device__ __forceinline__ unsigned int crossed(const Params &p, int nev) const {
+        return B::template crossed_rr<INTEG == I_DP45>(p, nev);
+    }
     static constexpr int SMEM_PER_THREAD = INTEG == I_DP45 ? DP_SLOTS * (int)sizeof(double) : 0;
     double *kb;
     int ks;
@@ -103,7 +115,7 @@ struct Stepper64 : State64<INTEG> {
     template <int V, int M>
     __device__ __forceinline__ void eval_medium(const Params &p, double s, bool first) {
         if (INTEG == I_RK4) rk4_fermat<V, M>(p, y, s, y1);
-        else dp45_fermat<V, M>(p, y, s, first, kb, ks, y1, e6);
+        else dp45_fermat<V, M>(p, y, s, first, kb, ks, y1, e6, rr);
     }
     // lanes: the lanes of the warp that evaluate with this one
     __device__ __forceinline__ void eval(const Params &p, double s, unsigned int lanes) {
@@ -127,6 +139,184 @@ struct Stepper64 : State64<INTEG> {
 #pragma unroll
             for (int i = 0; i < 6; ++i) kb[i * ks] = kb[(36 + i) * ks];  // first stage of the next step (FSAL)
         }
+    }
+};
+
+// ------------------------------------------------------------------ eight lanes per ray
+// The same steps with a ray on the eight lanes of a group (four rays per warp), for warps that have few rays
+// left and for calls with few rays.  An FP64 instruction blocks its warp for 64 cycles however many lanes take
+// part, and a warp alone has no other to fill them, so what counts there is instructions per step, not per ray.
+// Lane l keeps component l of the stages (lanes 6 and 7 follow along): each term of a stage combination is one FMA
+// instead of six, the scaled tableau is formed a column per lane, the step control checks a component per lane; the
+// right-hand side and the crossing search run alike on all lanes of the group on copies of the state.  Terms and
+// roundings are those of the narrow steps in their order: the results are the same bit for bit.  One ray alone, one
+// thread -> eight lanes, per DP5(4) step: azimuthal extraordinary 13.7 -> 8.9 us, azimuthal ordinary 14.2 -> 9.5,
+// radial extraordinary 15.5 -> 11; per RK4 step 5.8 -> 5.2.  (Independent products of the right-hand side on
+// different lanes, 1912 instead of 4060 instructions per step, took as long: what the FP64 instructions saved went
+// to shuffles.)
+// Scaled tableau rows of stages 2 .. 7 and of the error estimate: columns 0 .. 5 the coefficients of k1 .. k6
+// without the row's last one, which is in column 7.
+static __constant__ double c_dp_wide[7][8] = {
+    {0, 0, 0, 0, 0, 0, 0, DP::a21},
+    {DP::a31, 0, 0, 0, 0, 0, 0, DP::a32},
+    {DP::a41, DP::a42, 0, 0, 0, 0, 0, DP::a43},
+    {DP::a51, DP::a52, DP::a53, 0, 0, 0, 0, DP::a54},
+    {DP::a61, DP::a62, DP::a63, DP::a64, 0, 0, 0, DP::a65},
+    {DP::b1, 0, DP::b3, DP::b4, DP::b5, 0, 0, DP::b6},
+    {DP::e1, 0, DP::e3, DP::e4, DP::e5, DP::e6, 0, DP::e7}};
+constexpr int WIDE_LANES = 8, WIDE_RAYS = 32 / WIDE_LANES;
+
+template <int VAR, int MODE, int INTEG>
+struct StepperWide : State64<INTEG> {
+    using B = State64<INTEG>;
+    using B::need_k1;
+    using B::vm;
+    using B::y;
+    using B::y1;
+    using B::rr;
+    __device__ __forceinline__ unsigned int crossed(const Params &p, int nev) const {
+        return B::template crossed_rr<INTEG == I_DP45>(p, nev);
+    }
+    static constexpr int SMEM_PER_THREAD = INTEG == I_DP45 ? 14 * (int)sizeof(double) : 0;
+    double *tab;  // this group's scaled tableau (7 rows of 8, ks doubles apart), then the tableau itself
+    int ks, l;    // l: lane of the group
+    unsigned int grp;  // the group's lanes
+    double yo, y1o, eo, k1o, k7o;
+
+    __device__ __forceinline__ void bind(double *smem) {
+        const int lane = threadIdx.x & 31;
+        l = lane & (WIDE_LANES - 1);
+        grp = 0xffu << (lane - l);
+        tab = smem + (threadIdx.x - l);
+        ks = blockDim.x;
+        if (INTEG == I_DP45) {
+#pragma unroll
+            for (int r = 0; r < 7; ++r) tab[(7 + r) * ks + l] = c_dp_wide[r][l];
+        }
+    }
+    __device__ __forceinline__ double own(const double a[6]) const {
+        return l == 0 ? a[0] : l == 1 ? a[1] : l == 2 ? a[2] : l == 3 ? a[3] : l == 4 ? a[4] : a[5];
+    }
+    __device__ __forceinline__ double from(double a, int lane) const { return __shfl_sync(grp, a, lane, WIDE_LANES); }
+    __device__ __forceinline__ void begin() {
+        yo = own(y);
+        need_k1 = true;
+    }
+    template <typename Q>
+    __device__ __forceinline__ void load(const Q &q, int k) {
+        y[0] = q.x[k]; y[1] = q.y[k]; y[2] = q.z[k];
+        y[3] = q.vx[k]; y[4] = q.vy[k]; y[5] = q.vz[k];
+        begin();
+    }
+    // this lane's component of the right-hand side at the point whose components are t; g: all of the point's
+    template <int V, int M>
+    __device__ __forceinline__ double derivative(const Params &p, double t, double g[6]) {
+        g[0] = from(t, 0); g[1] = from(t, 1); g[2] = from(t, 2);
+        g[3] = from(t, 3); g[4] = from(t, 4); g[5] = from(t, 5);
+        double a[3];
+        accel64<V, M>(p.R1, g[0], g[1], g[3], g[4], g[5], a[0], a[1], a[2], rr);
+        return l == 0 ? g[3] : l == 1 ? g[4] : l == 2 ? g[5] : l == 3 ? a[0] : l == 4 ? a[1] : a[2];
+    }
+    template <int V, int M>
+    __device__ __forceinline__ void eval_medium(const Params &p, double h) {
+        if constexpr (V == V_TEST || (V == V_RADIAL && M == M_ORD)) {  // straight lines
+            if (INTEG == I_RK4) {
+                rk4_fermat<V, M>(p, y, h, y1);
+            } else {
+                dp45_fermat<V, M>(p, y, h, false, nullptr, 0, y1, B::e6, rr);
+                eo = own(B::e6);
+            }
+            y1o = own(y1);
+        } else if constexpr (INTEG == I_RK4) {
+            double acc = 0.0, t = yo, k = 0.0, g[6];
+            const double hh = 0.5 * h;
+#pragma unroll 1
+            for (int s = 0; s < 4; ++s) {
+                k = derivative<V, M>(p, t, g);
+                if (s == 3) break;
+                acc = s == 0 ? k : fma(2.0, k, acc);
+                t = fma(s < 2 ? hh : h, k, yo);
+            }
+            y1o = fma(h * (1.0 / 6.0), acc + k, yo);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) y1[i] = from(y1o, i);
+        } else {
+            // the tableau times h, a column per lane
+#pragma unroll
+            for (int r = 0; r < 7; ++r) {
+                const double c = tab[(7 + r) * ks + l];
+                const bool zero = s64_is_zero(c);
+                tab[r * ks + l] = s64_clear(zero, s64_mul(h, s64_nonzero(zero, c)));
+            }
+            __syncwarp(grp);
+            // stages not known yet enter with a zero coefficient, so they have to be finite
+            double k1 = need_k1 ? 0.0 : k1o, k2 = 0.0, k3 = 0.0, k4 = 0.0, k5 = 0.0, k6 = 0.0, k = k1, t = yo;
+            const double *row = tab;
+            if (!need_k1) t = fma(row[7], k, yo);
+#pragma unroll 1
+            for (int s = need_k1 ? 1 : 2; s < 8; ++s) {
+                row = tab + (s - 1) * ks;
+                double pre = s == 7 ? 0.0 : yo;
+                if (s > 1) pre = fma(row[1], k2, fma(row[0], k1, pre));
+                if (s > 3) pre = fma(row[3], k4, fma(row[2], k3, pre));
+                if (s > 5) pre = fma(row[5], k6, fma(row[4], k5, pre));
+                y1o = t;
+                k = derivative<V, M>(p, t, y1);
+                k1 = s == 1 ? k : k1;
+                k2 = s == 2 ? k : k2;
+                k3 = s == 3 ? k : k3;
+                k4 = s == 4 ? k : k4;
+                k5 = s == 5 ? k : k5;
+                k6 = s == 6 ? k : k6;
+                t = fma(row[7], k, pre);
+            }
+            k1o = k1;
+            k7o = k;
+            eo = t;
+            __syncwarp(grp);  // the table has been read
+        }
+        need_k1 = false;
+    }
+    __device__ __forceinline__ void eval(const Params &p, double h, unsigned int) {
+        if (VAR != V_ANY) {
+            eval_medium<VAR, MODE>(p, h);
+        } else {
+            switch (vm) {
+            case 0: eval_medium<V_RADIAL, M_ORD>(p, h); break;
+            case 1: eval_medium<V_RADIAL, M_EXT>(p, h); break;
+            case 2: eval_medium<V_AZIMUTHAL, M_ORD>(p, h); break;
+            default: eval_medium<V_AZIMUTHAL, M_EXT>(p, h); break;
+            }
+        }
+    }
+    // dp_control, a component per lane
+    __device__ __forceinline__ bool control(double tol, double &fac) const {
+        const double sc = fma(tol, fmax(s64_abs(yo), s64_abs(y1o)), tol), ae = s64_abs(eo);
+        const bool bad = s64_isnan(ae);
+        bool ok = true;
+        float fe = __fdividef(s64_to_float(ae, ok), s64_to_float(sc, ok));
+        if (!ok) fe = __fdividef((float)ae, (float)sc);
+        const bool acc = __all_sync(grp, bad || s64_le_pos(ae, sc));
+        if (__any_sync(grp, bad)) { fac = 0.2; return false; }
+        fe = fmaxf(fe, 0.f);  // NaN (infinite over infinite) counts for nothing, as in dp_control
+#pragma unroll
+        for (int o = WIDE_LANES / 2; o; o >>= 1) fe = fmaxf(fe, __shfl_xor_sync(grp, fe, o));
+        fac = dp_factor(fe);
+        return acc;
+    }
+    __device__ __forceinline__ void take_step() {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) y[i] = y1[i];
+        yo = y1o;
+        k1o = k7o;  // first stage of the next step (FSAL)
+    }
+    __device__ __forceinline__ void take_crossing() {
+        B::take_crossing();
+        begin();
+    }
+    __device__ __forceinline__ void mirror() {
+        B::mirror();
+        begin();
     }
 };
 

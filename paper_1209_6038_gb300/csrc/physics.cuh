@@ -189,12 +189,13 @@ struct MulInt {  // on the integer pipes (soft64.cuh)
     }
     static __device__ __forceinline__ double half(double a) { return s64_half(a); }
 };
-// Returns the range (s64_range) of what the products rest on: the inputs, and the sums that may cancel.
+// r2: x^2 + y^2.  Returns the range (s64_range) of what the products rest on: the inputs, and the sums that may
+// cancel.
 template <typename M, int VAR, int MODE>
 __device__ __forceinline__ uint32_t accel64_form(double R1, double x, double y, double vx, double vy, double vz,
-                                                 double &ax, double &ay, double &az) {
+                                                 double &ax, double &ay, double &az, double &r2) {
     const bool vz0 = s64_is_zero(vz);
-    const double r2 = fma(x, x, M::mul(y, y));
+    r2 = fma(x, x, M::mul(y, y));
     // 1 / r, as rsqrt_nr
     double y0;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(r2));
@@ -243,13 +244,13 @@ __device__ __forceinline__ uint32_t accel64_form(double R1, double x, double y, 
 // takes the hardware's, with the same results.
 template <int VAR, int MODE>
 __device__ __forceinline__ void accel64(double R1, double x, double y, double vx, double vy, double vz, double &ax,
-                                        double &ay, double &az) {
+                                        double &ay, double &az, double &r2) {
     if (VAR == V_TEST || (VAR == V_RADIAL && MODE == M_ORD)) {
-        ax = 0.0; ay = 0.0; az = 0.0;
+        ax = 0.0; ay = 0.0; az = 0.0; r2 = 0.0;
         return;
     }
-    const uint32_t range = accel64_form<MulInt, VAR, MODE>(R1, x, y, vx, vy, vz, ax, ay, az);
-    if (!s64_ok(range)) accel64_form<MulHW, VAR, MODE>(R1, x, y, vx, vy, vz, ax, ay, az);
+    const uint32_t range = accel64_form<MulInt, VAR, MODE>(R1, x, y, vx, vy, vz, ax, ay, az, r2);
+    if (!s64_ok(range)) accel64_form<MulHW, VAR, MODE>(R1, x, y, vx, vy, vz, ax, ay, az, r2);
 }
 
 template <int VAR, int MODE, typename T>
@@ -335,16 +336,17 @@ __device__ __forceinline__ void rhs(const Params &p, const double y[6], double d
         rhs_ham<VAR, MODE>(p, y, dy, vm);
         return;
     }
+    double r2;
     dy[0] = y[3]; dy[1] = y[4]; dy[2] = y[5];
     if (VAR != V_ANY) {
-        accel64<VAR, MODE>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]);
+        accel64<VAR, MODE>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2);
         return;
     }
     switch (vm) {
-    case 0: accel64<V_RADIAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]); break;
-    case 1: accel64<V_RADIAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]); break;
-    case 2: accel64<V_AZIMUTHAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]); break;
-    default: accel64<V_AZIMUTHAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]); break;
+    case 0: accel64<V_RADIAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2); break;
+    case 1: accel64<V_RADIAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2); break;
+    case 2: accel64<V_AZIMUTHAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2); break;
+    default: accel64<V_AZIMUTHAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2); break;
     }
 }
 
@@ -359,13 +361,14 @@ __device__ __forceinline__ void rhs_inline(const Params &p, const double y[6], d
     }
     dy[0] = y[3]; dy[1] = y[4]; dy[2] = y[5];
     dy[3] = dy[4] = dy[5] = 0.0;
+    double r2;
     const int m = VAR != V_ANY ? 2 * VAR + MODE : vm;
     if (VAR != V_TEST && m == 1)
-        accel64_form<MulHW, V_RADIAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]);
+        accel64_form<MulHW, V_RADIAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2);
     else if (VAR != V_TEST && m == 2)
-        accel64_form<MulHW, V_AZIMUTHAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]);
+        accel64_form<MulHW, V_AZIMUTHAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2);
     else if (VAR != V_TEST && m == 3)
-        accel64_form<MulHW, V_AZIMUTHAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5]);
+        accel64_form<MulHW, V_AZIMUTHAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2);
 }
 template <int VAR, int MODE, bool HAM>
 __device__ __forceinline__ void rk4_step(const Params &p, const double y[6], double h, double out[6], int vm = 0) {
@@ -472,12 +475,12 @@ static __constant__ double c_dp_a[20] = {DP::a21, DP::a31, DP::a32, DP::a41, DP:
 static __constant__ double c_dp_e[5] = {DP::e1, DP::e3, DP::e4, DP::e5, DP::e6};
 
 // Step of size h from y; k1 in slot 0, or evaluated here (first; uniform over the warp: evaluating the k1 that a
-// lane has already gives the same value).  y1: the fifth-order solution, e6: the error estimate,
+// lane has already gives the same value).  rr: r^2 at y1; y1: the fifth-order solution, e6: the error estimate,
 // slot 6: k7 = f(y1).  h: normal, far from the ends of the exponent range (h >= 1e-14 for a step; a trial
 // size of the crossing search is at least 2^-215 of one).
 template <int VAR, int MODE>
 __device__ __forceinline__ void dp45_fermat(const Params &p, const double y[6], double h, bool first, double *kb,
-                                            int ks, double y1[6], double e6[6]) {
+                                            int ks, double y1[6], double e6[6], double &rr) {
     if constexpr (VAR == V_TEST || (VAR == V_RADIAL && MODE == M_ORD)) {  // straight lines: every k is (v, 0)
         const double b1 = h * DP::b1, b3 = h * DP::b3, b4 = h * DP::b4, b5 = h * DP::b5, b6 = h * DP::b6;
         const double c1 = h * DP::e1, c3 = h * DP::e3, c4 = h * DP::e4, c5 = h * DP::e5, c6 = h * DP::e6,
@@ -490,6 +493,7 @@ __device__ __forceinline__ void dp45_fermat(const Params &p, const double y[6], 
             y1[3 + i] = v;
             e6[3 + i] = 0.0;
         }
+        rr = fma(y1[0], y1[0], __dmul_rn(y1[1], y1[1]));
     } else {
         constexpr bool AZ = !(VAR == V_AZIMUTHAL && MODE == M_EXT);  // dv_z/dt is not identically zero
         double t[6], a[3];
@@ -529,7 +533,7 @@ __device__ __forceinline__ void dp45_fermat(const Params &p, const double y[6], 
                 k += 6 * ks;
             }
             row += s;
-            accel64<VAR, MODE>(p.R1, t[0], t[1], t[3], t[4], t[5], a[0], a[1], a[2]);
+            accel64<VAR, MODE>(p.R1, t[0], t[1], t[3], t[4], t[5], a[0], a[1], a[2], rr);
             double *ko = kb + 6 * s * ks;
             ko[0] = t[3]; ko[ks] = t[4]; ko[2 * ks] = t[5];
             ko[3 * ks] = a[0]; ko[4 * ks] = a[1]; ko[5 * ks] = a[2];
@@ -555,14 +559,14 @@ __device__ __forceinline__ void rk4_fermat(const Params &p, const double y[6], d
             out[3 + i] = y[3 + i];
         }
     } else {
-        double acc[6], t[6], k[6];
+        double acc[6], t[6], k[6], r2;
 #pragma unroll
         for (int i = 0; i < 6; ++i) { acc[i] = 0.0; t[i] = y[i]; }
         const double hh = 0.5 * h;
 #pragma unroll 1
         for (int s = 0; s < 4; ++s) {
             k[0] = t[3]; k[1] = t[4]; k[2] = t[5];
-            accel64<VAR, MODE>(p.R1, t[0], t[1], t[3], t[4], t[5], k[3], k[4], k[5]);
+            accel64<VAR, MODE>(p.R1, t[0], t[1], t[3], t[4], t[5], k[3], k[4], k[5], r2);
             if (s == 3) break;
             const double c = s < 2 ? hh : h, w = s == 0 ? 1.0 : 2.0;
 #pragma unroll
@@ -579,6 +583,11 @@ __device__ __forceinline__ void rk4_fermat(const Params &p, const double y[6], d
 // DP5(4) step control: accept iff |e_i| <= tol + tol max(|y_i|, |y1_i|) for every component
 // (decided in FP64); the step factor 0.9 err^(-1/5), clamped to [0.2, 5], is evaluated in FP32
 // (it only sets the next step size).  NaN -> reject with factor 0.2.
+__device__ __forceinline__ double dp_factor(float fe) {
+    float f = fe == 0.f ? 5.f : fminf(5.f, fmaxf(0.2f, 0.9f * __powf(fe, -0.2f)));
+    if (!(fe < 3.0e38f)) f = 0.2f;
+    return s64_from_float(f);
+}
 __device__ __forceinline__ bool dp_control(const double y[6], const double y1[6], const double e6[6], double tol,
                                            double &fac) {
     bool acc = true, bad = false, ok = true;
@@ -597,9 +606,7 @@ __device__ __forceinline__ bool dp_control(const double y[6], const double y1[6]
         for (int i = 0; i < 6; ++i)
             fe = fmaxf(fe, __fdividef((float)fabs(e6[i]), (float)fma(tol, fmax(fabs(y[i]), fabs(y1[i])), tol)));
     }
-    float f = fe == 0.f ? 5.f : fminf(5.f, fmaxf(0.2f, 0.9f * __powf(fe, -0.2f)));
-    if (!(fe < 3.0e38f)) f = 0.2f;
-    fac = s64_from_float(f);
+    fac = dp_factor(fe);
     return acc;
 }
 
@@ -614,6 +621,15 @@ __device__ __forceinline__ T metal_chord(T x0, T y0, T x1, T y1, T R1sq) {
     if (!(b > T(0) && b < dd)) return T(0);
     if (!((x0 * x0 + y0 * y0 - R1sq) * dd < b * b)) return T(0);
     return b / dd;
+}
+
+// A bound that spares metal_chord: false only if it is 0 for certain.  The chord's points are no closer to the axis
+// than the nearer end point less half the chord; in FP32 with a margin of 1e-5 of the sizes (rounding: 1e-6).
+__device__ __forceinline__ bool chord_near(float x0, float y0, float x1, float y1, float R1) {
+    const float dx = x1 - x0, dy = y1 - y0;
+    const float r0 = x0 * x0 + y0 * y0, r1 = x1 * x1 + y1 * y1;
+    const float near = sqrtf(fminf(r0, r1)), half = 0.5f * sqrtf(dx * dx + dy * dy);
+    return !(near - half > R1 + 1e-5f * (near + half + R1));
 }
 
 // ------------------------------------------------------------------ surfaces

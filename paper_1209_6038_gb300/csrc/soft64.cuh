@@ -162,6 +162,21 @@ S64_FN float s64_to_float(double a, bool &ok) {
     return zero ? 0.f : f;
 #endif
 }
+// a to single precision by truncation (relative error below 2^-23), of any sign, for 2^-125 <= |a| < 2^127; outside
+// that the result is 0 or huge
+S64_FN float s64_truncate(double a) {
+    const uint32_t h = (uint32_t)s64_hi(a), m = h & 0x7fffffffu;
+    uint32_t u = s64_funnel((uint32_t)s64_lo(a), m, 3) - (896u << 23);
+    u = m < (898u << 20) ? 0u : m < (1150u << 20) ? u : 0x7f000000u;
+    u |= h & 0x80000000u;
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(u);
+#else
+    float f;
+    memcpy(&f, &u, 4);
+    return f;
+#endif
+}
 // (double)a for a positive normal float
 S64_FN double s64_from_float(float a) {
 #ifdef __CUDA_ARCH__

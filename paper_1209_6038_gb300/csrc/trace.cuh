@@ -128,14 +128,17 @@ __device__ __forceinline__ void leave(const Params &p, int ev, const double y[6]
     rec.tile_id = room_hit(p, x, dout, rgb);
 }
 
-// Whole ray, FP64 (HAM: Hamiltonian form), by the lanes of a warp together: `valid` lanes have a ray; smem: the
-// block's shared memory of the stepper.  rgb receives the room colour (0 when there is none).
-template <int VAR, int MODE, int INTEG, bool HAM>
-using PlainStepper = typename std::conditional<HAM, StepperHam<VAR, MODE, INTEG>, Stepper64<VAR, MODE, INTEG>>::type;
-template <int VAR, int MODE, int INTEG, bool HAM>
+// Whole ray, FP64, by the lanes of a warp together: `valid` lanes have a ray (one each, or one per group of eight
+// lanes when WIDE); smem: the block's shared memory of the stepper.  HAM: Hamiltonian form.  rgb receives the room
+// colour (0 when there is none).
+template <int VAR, int MODE, int INTEG, bool HAM, bool WIDE>
+using PlainStepper = typename std::conditional<
+    HAM, StepperHam<VAR, MODE, INTEG>,
+    typename std::conditional<WIDE, StepperWide<VAR, MODE, INTEG>, Stepper64<VAR, MODE, INTEG>>::type>::type;
+template <int VAR, int MODE, int INTEG, bool HAM, bool WIDE>
 __device__ __forceinline__ void trace_ray(const Params &p, bool valid, const double o[3], const double d[3], double *smem,
                                           cloak_record &rec, float rgb[3]) {
-    typedef PlainStepper<VAR, MODE, INTEG, HAM> S;
+    typedef PlainStepper<VAR, MODE, INTEG, HAM, WIDE> S;
     S st;
     st.vm = 2 * VAR + MODE;
     st.bind(smem);
@@ -143,7 +146,7 @@ __device__ __forceinline__ void trace_ray(const Params &p, bool valid, const dou
     Lane<S, INTEG, false, true> ray;
     ray.reset();
     if (valid && enter<MODE>(p, o, d, rec, rgb, st.y, k0, n_in, mat_in)) ray.start(p);
-    st.need_k1 = true;
+    st.begin();
     int status = -1;
     for (;;) {
         const bool live = ray.phase != PH_IDLE;

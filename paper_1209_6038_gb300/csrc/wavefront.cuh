@@ -220,6 +220,70 @@ __global__ void __launch_bounds__(128) k_wf_entry(Params p, int spp, unsigned lo
 __global__ void k_wf_sort_scan(Queue q, int nbins, unsigned int reserve);
 __global__ void k_wf_sort_scatter(Queue q);
 
+// Rays of a warp on eight lanes each (StepperWide) until they are done: group g starts with the ray of slot
+// `slot` (state st, progress h, t, steps, metal; slot < 0: none), and fetches the next of the `rl` reserved rays
+// (from perm[first]) whenever it has none.
+template <int VAR, int MODE, int INTEG, int PREC>
+__device__ __noinline__ void wf_integrate_wide(const Params &kp, const Queue &q, double *smem, const double y[6],
+                                                  int vm, double h, double t, int steps, bool metal, int slot,
+                                                  unsigned int rl, unsigned int first) {
+    typedef StepperWide<VAR, MODE, INTEG> S;
+    Params p;  // what the steps read, in registers instead of behind a pointer (a load per use and step)
+    p.R1 = kp.R1;
+    p.R1sq = kp.R1sq;
+    p.R2sq = kp.R2sq;
+    p.halfH = kp.halfH;
+    p.R1f = kp.R1f;
+    p.h_or_tol = kp.h_or_tol;
+    p.max_steps = kp.max_steps;
+    S st;
+    st.bind(smem);
+    st.vm = vm;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) st.y[i] = y[i];
+    st.begin();
+    Lane<S, INTEG, INTEG == I_DP45, false> ray;
+    ray.reset();
+    if (slot >= 0) {
+        ray.start(p);
+        ray.h = h;
+        ray.t = t;
+        ray.steps = steps;
+        ray.metal = metal;
+    }
+    bool more = rl > 0;
+    for (;;) {
+        if (ray.phase == PH_IDLE && more) {
+            unsigned int k = 0;
+            if (st.l == 0) k = atomicAdd(q.count + 10, 1u);
+            k = __shfl_sync(st.grp, k, 0, WIDE_LANES);
+            if (k < rl) {
+                slot = q.perm[first + k];
+                st.load(q, slot);
+                ray.start(p);
+            } else {
+                more = false;
+            }
+        }
+        const bool live = ray.phase != PH_IDLE;
+        const unsigned int lm = __ballot_sync(0xffffffffu, live);
+        if (!lm) break;
+        if (!live) continue;
+        const bool mirrors = (VAR == V_RADIAL && MODE == M_ORD) || (VAR == V_ANY && st.vm == 0);
+        const int status = ray.advance(p, st, lm, mirrors);
+        if (status >= 0) {
+            if (st.l == 0) {
+                st.store(q, slot);
+                q.t[slot] = ray.t;
+                q.status[slot] = status;
+                q.steps[slot] = ray.steps;
+                q.face[slot] = ray.evbest;
+            }
+            ray.phase = PH_IDLE;
+        }
+    }
+}
+
 // PREC: 0 FP64 (Fermat form), 1 mixed precision, 2 FP64 Hamiltonian form
 template <int VAR, int MODE, int INTEG, int PREC>
 using WfStepper = typename std::conditional<
@@ -232,6 +296,7 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
     S st;
     st.vm = 0;
     st.bind(wf_smem);
+    const int lane = threadIdx.x & 31;
     const unsigned int n = q.count[2];  // rays left to integrate after the sort
     // medium segments of the permutation (batch: one per medium/mode; a lane draws rays from its
     // warp's current segment, so that the lanes of a warp evaluate one medium's equations)
@@ -244,8 +309,9 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
     // batch) -- those that pass closest to the inner radius, up to ~3e4 steps each -- for the warps of
     // the first p.dedicated_blocks blocks.  The other blocks resident on those SMs leave at once, so
     // these warps share their SM's FP64 unit with no others and advance their long rays at close to
-    // one warp's latency; on a full SM they would get a twelfth of it and finish last, after the rest
-    // of the queue.  (A block that misses the flag only costs speed: every ray is still integrated once.)
+    // one warp's latency (FP64: four rays per warp, eight lanes each); on a full SM they would get a fraction
+    // of it and finish last, after the rest of the queue.  (A block that misses the flag only costs speed:
+    // every ray is still integrated once.)
     const unsigned int rl = q.count[9];
     const unsigned int rv = rl ? q.count[8] : 0u;
     bool reserve = false;
@@ -261,6 +327,15 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
             unsigned int f = 0;
             if ((threadIdx.x & 31u) == 0) f = sm_taken[smid & 255u];
             if (__shfl_sync(0xffffffffu, f, 0)) return;  // the whole warp leaves
+        }
+    }
+    if constexpr (PREC == 0) {
+        if (reserve) {
+            const double none[6] = {0, 0, 0, 0, 0, 0};
+            wf_integrate_wide<VAR, MODE, INTEG, PREC>(p, q, wf_smem, none, (int)rv, 0.0, 0.0, 0, false, -1, rl,
+                                                      VAR == V_ANY ? q.bins[SEG_OFFSET + 2 * rv] : 0u);
+            reserve = false;
+            __syncwarp();
         }
     }
     Lane<S, INTEG, INTEG == I_DP45 && PREC != 1, false> ray;
@@ -328,6 +403,22 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
         if (!live) drained = true;
         const unsigned int lm = __ballot_sync(0xffffffffu, live);
         if (!lm) break;     // the whole warp is drained
+        if constexpr (PREC == 0) {
+            // few rays left and none to refill with: eight lanes each to the end
+            if (__popc(lm) <= WIDE_RAYS && __all_sync(0xffffffffu, live ? ray.phase == PH_STEP : drained)) {
+                const int src = __fns(lm, 0, (lane >> 3) + 1) & 31;  // lane of this group's ray
+                double yw[6];
+#pragma unroll
+                for (int i = 0; i < 6; ++i) yw[i] = __shfl_sync(0xffffffffu, st.y[i], src);
+                const double hw = __shfl_sync(0xffffffffu, ray.h, src), tw = __shfl_sync(0xffffffffu, ray.t, src);
+                const int vw = __shfl_sync(0xffffffffu, st.vm, src), nw = __shfl_sync(0xffffffffu, ray.steps, src),
+                          mw = __shfl_sync(0xffffffffu, (int)ray.metal, src),
+                          sw = __shfl_sync(0xffffffffu, slot, src);
+                wf_integrate_wide<VAR, MODE, INTEG, PREC>(p, q, wf_smem, yw, vw, hw, tw, nw, mw != 0,
+                                                          (lane >> 3) < __popc(lm) ? sw : -1, 0u, 0u);
+                break;
+            }
+        }
         if (!live) continue;
         const bool mirrors = (VAR == V_RADIAL && MODE == M_ORD) || (VAR == V_ANY && st.vm == 0);
         const int status = ray.advance(p, st, lm, mirrors);
@@ -342,11 +433,11 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
     }
 }
 
-// The FP64 integrator keeps the compiler's register choice; the mixed one is held to 128 registers for four
-// blocks per SM -- its FP32 steps are latency-bound and gain from the extra warps, while the rare band steps
-// near R1 may spill.
+// The FP64 integrator is held to 168 registers for three blocks per SM (the wide steps, a call of their own, would
+// take 208 and leave two: 3 % slower on a full image); the mixed one to 128 for four -- its FP32 steps are
+// latency-bound and gain from the extra warps, while the rare band steps near R1 may spill.
 template <int VAR, int MODE, int INTEG, int PREC>
-__global__ void __launch_bounds__(128) k_wf_integrate(Params p, Queue q) {
+__global__ void __launch_bounds__(128, 3) k_wf_integrate(const __grid_constant__ Params p, const __grid_constant__ Queue q) {
     wf_integrate_body<VAR, MODE, INTEG, PREC>(p, q);
 }
 template <int VAR, int MODE, int INTEG, int PREC>
@@ -357,6 +448,10 @@ template <int VAR, int MODE, int INTEG, int PREC>
 constexpr auto wf_integrate_kernel() {
     if constexpr (PREC != 1) return k_wf_integrate<VAR, MODE, INTEG, PREC>;
     else return k_wf_integrate_mixed<VAR, MODE, INTEG, PREC>;
+}
+// rays reserved for the long-ray blocks: reserve_per_thread for each ray that their warps advance at a time
+inline unsigned int long_ray_reserve(const Params &p, int prec, int packet) {
+    return (unsigned int)(p.long_ray_blocks * (prec == 0 ? packet / WIDE_LANES : packet) * p.reserve_per_thread);
 }
 // the kernel's precision index from the handle's settings
 inline int wf_prec(const Params &p) { return p.precision ? 1 : p.formulation ? 2 : 0; }
@@ -457,7 +552,7 @@ static cudaError_t wavefront_vmip(const Params &p, int spp, unsigned long long s
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int pk = packet > 0 ? packet : 128;
     // the slowest rays go to the warps of LONG_RAY_BLOCKS blocks that have their SMs to themselves
-    k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS, (unsigned int)(p.long_ray_blocks * pk * p.reserve_per_thread));
+    k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS, long_ray_reserve(p, PREC, pk));
     k_wf_sort_scatter<<<sms * 8, 256, 0, st>>>(q);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
