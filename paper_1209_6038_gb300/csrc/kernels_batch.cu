@@ -17,13 +17,21 @@ __global__ void __launch_bounds__(128) k_batch_entry(Params p, const ViewDev *vi
     long long local = g - vw.ray_begin, pix = local / spp;
     int s = (int)(local - pix * spp);
     int i = (int)(pix % vw.W), j = (int)(pix / vw.W);
+    float rgb[3];
+    if (!p.tof) {  // rays that miss, in single precision
+        const uint64_t px = uint64_t(j) * uint64_t(vw.W) + uint64_t(i);
+        const float xi1 = spp > 1 ? jitter_f32(seed, px, s, 0) : 0.5f, xi2 = spp > 1 ? jitter_f32(seed, px, s, 1) : 0.5f;
+        if (miss_f32(p, frame_f32(vw.eye, vw.fw, vw.rt, vw.up, vw.tx, vw.ty, vw.W, vw.Hp), i, j, xi1, xi2, rgb)) {
+            store_missed(p, samples, g, rgb);
+            return;
+        }
+    }
     double o[3], d[3], y[6], k0[3], n_in[3], mat[5];
     view_camera_ray(vw, i, j, s, spp, seed, o, d);
     Params pv = p;
     pv.variant = vw.vm >> 1;
     const int mode = vw.vm & 1;
     cloak_record rec;
-    float rgb[3];
     bool inside = mode ? enter<M_EXT>(pv, o, d, rec, rgb, y, k0, n_in, mat)
                        : enter<M_ORD>(pv, o, d, rec, rgb, y, k0, n_in, mat);
     if (!inside) {

@@ -97,6 +97,12 @@ __device__ __forceinline__ void store_sample(float4 *samples, cloak_record *recs
     if (recs) recs[id] = rec;
 }
 
+// Sample of a camera ray that misses the cylinder (enter): the room's colour, half of the light through a polariser.
+__device__ __forceinline__ void store_missed(const Params &p, float4 *samples, long long id, const float rgb[3]) {
+    const float w = p.analyzer ? 0.5f : 1.0f;
+    samples[id] = make_float4(w * rgb[0], w * rgb[1], w * rgb[2], w);
+}
+
 // Per-sample output of a TOF difference render (Params::tof): (w dt, w, 0, 0).
 __device__ __forceinline__ void store_tof_sample(const Params &p, float4 *samples, long long id, const double o[3],
                                                  const double d[3], const cloak_record &rec) {
@@ -196,10 +202,18 @@ __global__ void __launch_bounds__(128) k_wf_entry(Params p, int spp, unsigned lo
     long long pix = idx / spp;
     int s = (int)(idx - pix * spp);
     int i = (int)(pix % p.W), j = (int)(pix / p.W);
+    float rgb[3];
+    if (!recs) {  // rays that miss, in single precision (records carry their FP64 direction)
+        const uint64_t px = uint64_t(j) * uint64_t(p.W) + uint64_t(i);
+        const float xi1 = spp > 1 ? jitter_f32(seed, px, s, 0) : 0.5f, xi2 = spp > 1 ? jitter_f32(seed, px, s, 1) : 0.5f;
+        if (miss_f32(p, frame_f32(p.eye, p.fw, p.rt, p.up, p.tx, p.ty, p.W, p.Hp), i, j, xi1, xi2, rgb)) {
+            store_missed(p, samples, idx, rgb);
+            return;
+        }
+    }
     double o[3], d[3], y[6], k0[3], n_in[3], mat[5];
     camera_ray(p, i, j, s, spp, seed, o, d);
     cloak_record rec;
-    float rgb[3];
     if (!enter<MODE>(p, o, d, rec, rgb, y, k0, n_in, mat)) {
         store_sample(samples, recs, idx, rec, rgb);
         return;
