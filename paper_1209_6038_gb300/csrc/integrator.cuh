@@ -534,14 +534,24 @@ __device__ __forceinline__ void rk4_step_df(df R1, const df y[6], df h, df out[6
 // The band's steps near R1 (FP64 or double-float), out of line: rare, large, and kept out of the
 // instruction stream of the FP32 steps.  Inputs and outputs pass through the caller's local memory.
 template <int VAR, int MODE, int INTEG>
+__device__ __forceinline__ void band_medium_f64(const Params &p, const double *y, double s, double *yo, double *e,
+                                                double *kb, int ks) {
+    double rr;
+    if (INTEG == I_RK4) rk4_fermat<VAR, MODE>(p, y, s, yo);
+    else dp45_fermat<VAR, MODE>(p, y, s, true, kb, ks, yo, e, rr);
+}
+template <int VAR, int MODE, int INTEG>
 __device__ __noinline__ void band_step_f64(const Params &p, const double *y, double s, double *yo, double *e,
-                                           double *k7, int vm) {
-    if (INTEG == I_RK4) {
-        rk4_step<VAR, MODE, false>(p, y, s, yo, vm);
+                                           double *kb, int ks, int vm) {
+    if (VAR != V_ANY) {
+        band_medium_f64<VAR, MODE, INTEG>(p, y, s, yo, e, kb, ks);
     } else {
-        double k1[6];
-        rhs_inline<VAR, MODE, false>(p, y, k1, vm);
-        dp45_step<VAR, MODE, false>(p, y, k1, s, yo, e, k7, vm);
+        switch (vm) {
+        case 0: band_medium_f64<V_RADIAL, M_ORD, INTEG>(p, y, s, yo, e, kb, ks); break;
+        case 1: band_medium_f64<V_RADIAL, M_EXT, INTEG>(p, y, s, yo, e, kb, ks); break;
+        case 2: band_medium_f64<V_AZIMUTHAL, M_ORD, INTEG>(p, y, s, yo, e, kb, ks); break;
+        default: band_medium_f64<V_AZIMUTHAL, M_EXT, INTEG>(p, y, s, yo, e, kb, ks); break;
+        }
     }
 }
 template <int VAR, int MODE>
@@ -577,14 +587,19 @@ template <int VAR, int MODE, int INTEG>
 struct StepperMixed {
     typedef float real;
     static constexpr bool FP64 = false;
-    static constexpr int SMEM_PER_THREAD = 0;
+    static constexpr int SMEM_PER_THREAD = INTEG == I_DP45 ? DP_SLOTS * (int)sizeof(double) : 0;  // the FP64 band's stages
+    double *kb;
+    int ks;
     float yh[6], yl[6], k1[6];  // state (float-float) and first stage
     float y1h[6], y1l[6], e6[6], k7[6];
     float n6[6];  // rounding bound of the FP32 error estimate (noise floor)
     bool need_k1;
     int vm;  // 2 * variant + mode when VAR = MODE = V_ANY
 
-    __device__ __forceinline__ void bind(double *) {}
+    __device__ __forceinline__ void bind(double *smem) {
+        kb = smem + threadIdx.x;
+        ks = blockDim.x;
+    }
     // the queue holds the mixed path's states as float-float pairs: no conversion
     template <typename Q>
     __device__ __forceinline__ void load(const Q &q, int k) {
@@ -634,15 +649,15 @@ struct StepperMixed {
             return;
         }
         if (island(p)) {  // FP64 step from the float-float state
-            double y[6], yo[6], e[6], kk7[6];
+            double y[6], yo[6], e[6];
 #pragma unroll
             for (int i = 0; i < 6; ++i) y[i] = (double)yh[i] + (double)yl[i];
-            band_step_f64<VAR, MODE, INTEG>(p, y, (double)s, yo, e, kk7, vm);
+            band_step_f64<VAR, MODE, INTEG>(p, y, (double)s, yo, e, kb, ks, vm);
 #pragma unroll
             for (int i = 0; i < 6; ++i) {
                 y1h[i] = (float)yo[i];
                 y1l[i] = (float)(yo[i] - (double)y1h[i]);
-                if (INTEG == I_DP45) { e6[i] = (float)e[i]; k7[i] = (float)kk7[i]; n6[i] = 0.f; }
+                if (INTEG == I_DP45) { e6[i] = (float)e[i]; n6[i] = 0.f; }
             }
             need_k1 = true;
             return;
