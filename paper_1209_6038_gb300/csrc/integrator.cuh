@@ -462,58 +462,6 @@ __device__ __forceinline__ void rhs_df(df R1, const df y[6], df d[6], int vm) {
     }
 }
 template <int VAR, int MODE>
-__device__ __forceinline__ void dp45_step_df(df R1, const df y[6], const df k1[6], df h, df out[6], df err[6],
-                                             df k7[6], int vm) {
-    df k2[6], k3[6], k4[6], k5[6], k6[6], t[6];
-    {
-        const df c1 = h * df(DP::a21);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) t[i] = df_fma(c1, k1[i], y[i]);
-    }
-    rhs_df<VAR, MODE>(R1, t, k2, vm);
-    {
-        const df c1 = h * df(DP::a31), c2 = h * df(DP::a32);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) t[i] = df_fma(c2, k2[i], df_fma(c1, k1[i], y[i]));
-    }
-    rhs_df<VAR, MODE>(R1, t, k3, vm);
-    {
-        const df c1 = h * df(DP::a41), c2 = h * df(DP::a42), c3 = h * df(DP::a43);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) t[i] = df_fma(c3, k3[i], df_fma(c2, k2[i], df_fma(c1, k1[i], y[i])));
-    }
-    rhs_df<VAR, MODE>(R1, t, k4, vm);
-    {
-        const df c1 = h * df(DP::a51), c2 = h * df(DP::a52), c3 = h * df(DP::a53), c4 = h * df(DP::a54);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) t[i] = df_fma(c4, k4[i], df_fma(c3, k3[i], df_fma(c2, k2[i], df_fma(c1, k1[i], y[i]))));
-    }
-    rhs_df<VAR, MODE>(R1, t, k5, vm);
-    {
-        const df c1 = h * df(DP::a61), c2 = h * df(DP::a62), c3 = h * df(DP::a63), c4 = h * df(DP::a64),
-                 c5 = h * df(DP::a65);
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-            t[i] = df_fma(c5, k5[i], df_fma(c4, k4[i], df_fma(c3, k3[i], df_fma(c2, k2[i], df_fma(c1, k1[i], y[i])))));
-    }
-    rhs_df<VAR, MODE>(R1, t, k6, vm);
-    {
-        const df c1 = h * df(DP::b1), c3 = h * df(DP::b3), c4 = h * df(DP::b4), c5 = h * df(DP::b5),
-                 c6 = h * df(DP::b6);
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-            out[i] = df_fma(c6, k6[i], df_fma(c5, k5[i], df_fma(c4, k4[i], df_fma(c3, k3[i], df_fma(c1, k1[i], y[i])))));
-    }
-    rhs_df<VAR, MODE>(R1, out, k7, vm);
-    {
-        const df c1 = h * df(DP::e1), c3 = h * df(DP::e3), c4 = h * df(DP::e4), c5 = h * df(DP::e5),
-                 c6 = h * df(DP::e6), c7 = h * df(DP::e7);
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-            err[i] = df_fma(c7, k7[i], df_fma(c6, k6[i], df_fma(c5, k5[i], df_fma(c4, k4[i], df_fma(c3, k3[i], c1 * k1[i])))));
-    }
-}
-template <int VAR, int MODE>
 __device__ __forceinline__ void rk4_step_df(df R1, const df y[6], df h, df out[6], int vm) {
     df k[6], acc[6], t[6];
     const df hh = h * 0.5f, h6 = h * df(1.0 / 6.0);
@@ -554,32 +502,89 @@ __device__ __noinline__ void band_step_f64(const Params &p, const double *y, dou
         }
     }
 }
+// a double constant as a double-float pair
+#define CK_DF2(c) {(float)(c), (float)((c) - (double)(float)(c))}
+// The tableau in double-float (c_dp_a, c_dp_e of the FP64 form)
+static __constant__ float2 c_dp_a_df[20] = {CK_DF2(DP::a21), CK_DF2(DP::a31), CK_DF2(DP::a32), CK_DF2(DP::a41),
+                                            CK_DF2(DP::a42), CK_DF2(DP::a43), CK_DF2(DP::a51), CK_DF2(DP::a52),
+                                            CK_DF2(DP::a53), CK_DF2(DP::a54), CK_DF2(DP::a61), CK_DF2(DP::a62),
+                                            CK_DF2(DP::a63), CK_DF2(DP::a64), CK_DF2(DP::a65), CK_DF2(DP::b1),
+                                            CK_DF2(DP::b3),  CK_DF2(DP::b4),  CK_DF2(DP::b5),  CK_DF2(DP::b6)};
+static __constant__ float2 c_dp_e_df[5] = {CK_DF2(DP::e1), CK_DF2(DP::e3), CK_DF2(DP::e4), CK_DF2(DP::e5),
+                                           CK_DF2(DP::e6)};
+__device__ __forceinline__ df df_of(float2 v) { return df(v.x, v.y); }
+// DP5(4) step of one medium from y, its first stage included: the stages in shared memory (kb: this thread's
+// column, ks threads per row) and one copy of the right-hand side in a loop over them, as in dp45_fermat, because
+// the seven inlined copies of the unrolled form (3500 instructions per medium) left the mixed kernel's warps
+// waiting for instructions.
 template <int VAR, int MODE>
-__device__ __forceinline__ void dp45_band_df(df R1, const df *y, df hs, df *yo, df *e, df *k7, int vm) {
-    df k1[6];
-    rhs_df<VAR, MODE>(R1, y, k1, vm);
-    dp45_step_df<VAR, MODE>(R1, y, k1, hs, yo, e, k7, vm);
+__device__ __forceinline__ void dp45_band_df(df R1, const df *y, df h, df *yo, df *e, float2 *kb, int ks) {
+    const df unused;
+    if constexpr (VAR == V_TEST || (VAR == V_RADIAL && MODE == M_ORD)) {  // straight lines: no band (island)
+#pragma unroll
+        for (int i = 0; i < 6; ++i) { yo[i] = y[i]; e[i] = unused; }
+    } else {
+        df t[6], a[3];
+        int row = 0;
+#pragma unroll 1
+        for (int s = 0; s < 7; ++s) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) t[i] = y[i];
+            const int terms = s < 6 ? s : 5;
+            const float2 *k = kb;
+#pragma unroll 1
+            for (int q = 0; q < terms; ++q) {
+                const df c = h * df_of(c_dp_a_df[row + q]);
+                df kq[6];
+#pragma unroll
+                for (int i = 0; i < 6; ++i) kq[i] = df_of(k[i * ks]);
+                t[0] = df_fma(c, kq[0], t[0]);
+                t[1] = df_fma(c, kq[1], t[1]);
+#pragma unroll
+                for (int i = 3; i < 6; ++i) t[i] = df_fma(c, kq[i], t[i]);
+                if (s == 6) {
+                    const df ce = h * df_of(c_dp_e_df[q]);
+                    t[2] = df_fma(c, kq[2], t[2]);
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) e[i] = q == 0 ? ce * kq[i] : df_fma(ce, kq[i], e[i]);
+                    if (q == 0) k += 6 * ks;  // no second stage in the solution
+                }
+                k += 6 * ks;
+            }
+            row += s;
+            accel_fixed<VAR, MODE, df>(R1, unused, unused, t[0], t[1], t[3], t[4], t[5], a[0], a[1], a[2]);
+            float2 *ko = kb + 6 * s * ks;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                ko[i * ks] = make_float2(t[3 + i].hi, t[3 + i].lo);
+                ko[(3 + i) * ks] = make_float2(a[i].hi, a[i].lo);
+            }
+        }
+        const df c7 = h * df(DP::e7);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) yo[i] = t[i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            e[i] = df_fma(c7, t[3 + i], e[i]);
+            e[3 + i] = df_fma(c7, a[i], e[3 + i]);
+        }
+    }
 }
 template <int VAR, int MODE, int INTEG>
-__device__ __noinline__ void band_step_df(float R1h, float R1l, const df *y, float s, df *yo, df *e, df *k7, int vm) {
+__device__ __noinline__ void band_step_df(float R1h, float R1l, const df *y, float s, df *yo, df *e, float2 *kb, int ks,
+                                          int vm) {
     const df R1(R1h, R1l), hs(s, 0.f);
-    if (VAR == V_ANY && INTEG == I_DP45) {
-        // the batch's medium chosen once per step: each medium's step with its right-hand sides inline
-        // (a call per stage cost the double-float step 5 % of its integration)
-        switch (vm) {
-        case 0: dp45_band_df<V_RADIAL, M_ORD>(R1, y, hs, yo, e, k7, vm); break;
-        case 1: dp45_band_df<V_RADIAL, M_EXT>(R1, y, hs, yo, e, k7, vm); break;
-        case 2: dp45_band_df<V_AZIMUTHAL, M_ORD>(R1, y, hs, yo, e, k7, vm); break;
-        default: dp45_band_df<V_AZIMUTHAL, M_EXT>(R1, y, hs, yo, e, k7, vm); break;
-        }
-        return;
-    }
     if (INTEG == I_RK4) {
         rk4_step_df<VAR, MODE>(R1, y, hs, yo, vm);
+    } else if (VAR == V_ANY) {  // the batch's medium chosen once per step
+        switch (vm) {
+        case 0: dp45_band_df<V_RADIAL, M_ORD>(R1, y, hs, yo, e, kb, ks); break;
+        case 1: dp45_band_df<V_RADIAL, M_EXT>(R1, y, hs, yo, e, kb, ks); break;
+        case 2: dp45_band_df<V_AZIMUTHAL, M_ORD>(R1, y, hs, yo, e, kb, ks); break;
+        default: dp45_band_df<V_AZIMUTHAL, M_EXT>(R1, y, hs, yo, e, kb, ks); break;
+        }
     } else {
-        df k1[6];
-        rhs_df<VAR, MODE>(R1, y, k1, vm);
-        dp45_step_df<VAR, MODE>(R1, y, k1, hs, yo, e, k7, vm);
+        dp45_band_df<VAR, MODE>(R1, y, hs, yo, e, kb, ks);
     }
 }
 
@@ -587,7 +592,7 @@ template <int VAR, int MODE, int INTEG>
 struct StepperMixed {
     typedef float real;
     static constexpr bool FP64 = false;
-    static constexpr int SMEM_PER_THREAD = INTEG == I_DP45 ? DP_SLOTS * (int)sizeof(double) : 0;  // the FP64 band's stages
+    static constexpr int SMEM_PER_THREAD = INTEG == I_DP45 ? DP_SLOTS * (int)sizeof(double) : 0;  // the band's stages
     double *kb;
     int ks;
     float yh[6], yl[6], k1[6];  // state (float-float) and first stage
@@ -634,14 +639,14 @@ struct StepperMixed {
     }
     __device__ __forceinline__ void eval(const Params &p, float s, unsigned int) {
         if (p.band_df && island(p)) {  // double-float step from the float-float state
-            df y[6], yo[6], e[6], kk7[6];
+            df y[6], yo[6], e[6];
 #pragma unroll
             for (int i = 0; i < 6; ++i) y[i] = df(yh[i], yl[i]);
             const df R1(p.R1);
-            band_step_df<VAR, MODE, INTEG>(R1.hi, R1.lo, y, s, yo, e, kk7, vm);
+            band_step_df<VAR, MODE, INTEG>(R1.hi, R1.lo, y, s, yo, e, reinterpret_cast<float2 *>(kb), ks, vm);
             if (INTEG == I_DP45) {
 #pragma unroll
-                for (int i = 0; i < 6; ++i) { e6[i] = e[i].hi + e[i].lo; k7[i] = kk7[i].hi; n6[i] = 0.f; }
+                for (int i = 0; i < 6; ++i) { e6[i] = e[i].hi + e[i].lo; n6[i] = 0.f; }
             }
 #pragma unroll
             for (int i = 0; i < 6; ++i) { y1h[i] = yo[i].hi; y1l[i] = yo[i].lo; }

@@ -473,8 +473,7 @@ inline int wf_prec(const Params &p) { return p.precision ? 1 : p.formulation ? 2
 template <int VAR, int MODE, int INTEG, int PREC>
 cudaError_t launch_wf_integrate(const Params &p, const Queue &q, int packet, int sms, cudaStream_t st) {
     constexpr auto kern = wf_integrate_kernel<VAR, MODE, INTEG, PREC>();
-    // (the double-float band keeps its stages elsewhere)
-    const size_t smem = PREC == 1 && p.band_df ? 0 : (size_t)WfStepper<VAR, MODE, INTEG, PREC>::SMEM_PER_THREAD * packet;
+    const size_t smem = (size_t)WfStepper<VAR, MODE, INTEG, PREC>::SMEM_PER_THREAD * packet;
     int nb = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, packet, smem);
     if (e != cudaSuccess) return e;
