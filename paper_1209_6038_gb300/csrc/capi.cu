@@ -97,6 +97,9 @@ static int make_params(const cloak *h, ck::Params &p) {
     p.R1x2 = 2.0 * h->R1;
     p.R1sq = h->R1 * h->R1;
     p.R2sq = h->R2 * h->R2;
+    p.gtol_lat = ck::CROSS_G_TOL * p.R2sq;
+    p.gtol_cap = ck::CROSS_G_TOL * p.halfH;
+    p.gtol_metal = ck::CROSS_G_TOL * p.R1sq;
     p.eo_t = h->eo_t;
     p.ee_t = h->ee_t;
     double cl = std::sqrt(h->c_t[0] * h->c_t[0] + h->c_t[1] * h->c_t[1] + h->c_t[2] * h->c_t[2]);

@@ -41,6 +41,7 @@ struct State64 {
     }
     __device__ __forceinline__ double g_start(const Params &p, int ev) const { return event_g(p, ev, y); }
     __device__ __forceinline__ double g_end(const Params &p, int ev) const { return event_g(p, ev, y1); }
+    __device__ __forceinline__ double g_end_rr(const Params &p, int ev) const { return event_g(p, ev, rr, y1[2]); }
     double rr;  // r^2 at y1, where the step leaves it (DP5(4) of the Fermat form)
     // surfaces behind the end point: bit ev is set iff event_g(ev, y1) > 0, decided by integer comparisons
     template <bool RR>
@@ -92,6 +93,9 @@ struct Stepper64 : State64<INTEG> {
     using B::rr;
     __device__ __forceinline__ unsigned int crossed(const Params &p, int nev) const {
         return B::template crossed_rr<INTEG == I_DP45>(p, nev);
+    }
+    __device__ __forceinline__ double g_end(const Params &p, int ev) const {
+        return INTEG == I_DP45 ? B::g_end_rr(p, ev) : B::g_end(p, ev);
     }
     static constexpr int SMEM_PER_THREAD = INTEG == I_DP45 ? DP_SLOTS * (int)sizeof(double) : 0;
     double *kb;
@@ -176,6 +180,9 @@ struct StepperWide : State64<INTEG> {
     using B::rr;
     __device__ __forceinline__ unsigned int crossed(const Params &p, int nev) const {
         return B::template crossed_rr<INTEG == I_DP45>(p, nev);
+    }
+    __device__ __forceinline__ double g_end(const Params &p, int ev) const {
+        return INTEG == I_DP45 ? B::g_end_rr(p, ev) : B::g_end(p, ev);
     }
     static constexpr int SMEM_PER_THREAD = INTEG == I_DP45 ? 14 * (int)sizeof(double) : 0;
     double *tab;  // this group's scaled tableau (7 rows of 8, ks doubles apart), then the tableau itself
@@ -847,6 +854,15 @@ __device__ __forceinline__ bool positive(double a) { return s64_positive(a); }
 __device__ __forceinline__ bool positive(float a) { return a > 0.f; }
 __device__ __forceinline__ bool le_pos(double a, double b) { return s64_le_pos(a, b); }  // 0 <= a or NaN, 0 <= b
 __device__ __forceinline__ bool le_pos(float a, float b) { return a <= b; }
+__device__ __forceinline__ bool not_positive(double a) { return s64_not_positive(a); }
+__device__ __forceinline__ bool not_positive(float a) { return a <= 0.f; }
+__device__ __forceinline__ bool not_negative(double a) { return s64_not_negative(a); }
+__device__ __forceinline__ bool not_negative(float a) { return a >= 0.f; }
+__device__ __forceinline__ bool same(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+__device__ __forceinline__ bool same(float a, float b) { return a == b; }
+// a <= f b for sizes a, b >= 0 whose ratio is decided to single precision
+__device__ __forceinline__ bool below(double a, float f, double b) { return s64_truncate(a) <= f * s64_truncate(b); }
+__device__ __forceinline__ bool below(float a, float f, float b) { return a <= f * b; }
 __device__ __forceinline__ double mag(double a) { return s64_abs(a); }
 __device__ __forceinline__ float mag(float a) { return fabsf(a); }
 
@@ -860,7 +876,7 @@ __device__ __forceinline__ float mag(float a) { return fabsf(a); }
 template <typename S, int INTEG, bool NEWTON, bool EXACT>
 struct Lane {
     typedef typename S::real R;
-    static constexpr double NEWTON_LAST = 1e-6;
+    static constexpr float NEWTON_LAST = 1e-6f;
     static constexpr int prefix = bisect_prefix<INTEG>();
     R h, t;
     int steps, phase;
@@ -892,7 +908,7 @@ struct Lane {
     __device__ __forceinline__ int advance(const Params &p, S &st, unsigned int lanes, bool mirrors) {
         const int nev = p.R1 > 0.0 ? 4 : 3;
         const R tol = (R)p.h_or_tol;
-        const R conv = sizeof(R) == 8 ? (R)CROSS_REL_TOL : (R)2.4e-7;  // bracket resolution of the search
+        const float conv = sizeof(R) == 8 ? (float)CROSS_REL_TOL : 2.4e-7f;  // bracket resolution of the search
         int status = -1;
         if (phase == PH_STEP && (steps >= p.max_steps || (INTEG == I_DP45 && !le_pos((R)1e-14, h))))
             status = CLOAK_RAY_STEP_LIMIT;
@@ -933,21 +949,26 @@ struct Lane {
                     t += h;
                     h *= fac;
                 } else {
-                    #pragma unroll
-                    for (int e = 0; e < 4; ++e) g1[e] = st.g_end(p, e);
+                                        // the values at the end point, of the further surfaces only if there are any
+                    ghi = st.g_end(p, __ffs(pending) - 1);
+                    g1[0] = ghi;
+                    if (pending & (pending - 1)) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) g1[e] = st.g_end(p, e);
+                    }
                     hs = h;
                     sbest = (R)1e30;
                     evbest = -1;
                     newton = false;
                     fin = false;
-                    search(p, st);
+                    search(p, st, ghi);
                     if (NEWTON) {
                         const R d0 = (R)st.g_rate_start(ev), d1 = (R)st.g_rate(ev);
-                        if (d0 >= (R)0 && d1 > (R)0) {
+                        if (not_negative(d0) && positive(d1)) {
                             newton = true;
-                            R s0 = hs - ghi / d1;
-                            if (!(s0 > (R)0 && s0 < hs)) s0 = hs * (-glo / (ghi - glo));
-                            if (!(s0 > (R)0 && s0 < hs)) s0 = (R)0.5 * hs;
+                            R s0 = fma(-ghi, rcp_nr(d1), hs);
+                            if (!inside(s0, (R)0, hs)) s0 = hs * (-glo / (ghi - glo));
+                            if (!inside(s0, (R)0, hs)) s0 = (R)0.5 * hs;
                             snext = s0;
                         }
                     }
@@ -956,7 +977,7 @@ struct Lane {
             }
         } else if (phase == PH_CROSS) {
             bool done = false;
-            const R gtol = (R)CROSS_G_TOL * (R)cross_g_scale(p, ev);
+            const R gtol = (R)cross_g_tol(p, ev);
             if (!inside(s, lo, hi)) {
                 done = true;
             } else if (NEWTON && newton) {
@@ -972,11 +993,11 @@ struct Lane {
                     done = true;
                 } else {
                     const R dg = (R)st.g_rate(ev);
-                    R sn = s - gs * rcp_nr(dg);
+                    R sn = fma(-gs, rcp_nr(dg), s);
                     if (!inside(sn, lo, hi)) sn = (R)0.5 * (lo + hi);
-                    else if (le_pos(mag(sn - s), (R)NEWTON_LAST * hs)) fin = true;
+                    else if (below(mag(sn - s), NEWTON_LAST, hs)) fin = true;
                     snext = sn;
-                    if (hi - lo <= conv * hi || it >= 100) done = true;
+                    if (below(hi - lo, conv, hi) || it >= 100) done = true;
                 }
             } else {
                 R gs = st.g_end(p, ev);
@@ -992,7 +1013,7 @@ struct Lane {
                     side = -1;
                 }
                 ++it;
-                if (it >= prefix && hi - lo <= conv * hi) done = true;
+                if (it >= prefix && below(hi - lo, conv, hi)) done = true;
                 // or a regula falsi trial point lies on the surface to rounding (Illinois approaches
                 // the root from one side, so the far end of the bracket may lag for many iterations)
                 if (!done && it > prefix && le_pos(mag(gs), gtol)) {
@@ -1004,12 +1025,13 @@ struct Lane {
             }
             if (done) {
                 R se = ev == EV_METAL ? lo : hi;
-                if (se < sbest) { sbest = se; evbest = ev; }
+                if (inside(se, (R)-1, sbest)) { sbest = se; evbest = ev; }
                 pending &= ~(1u << ev);
                 if (pending) {
                     newton = false;  // the coarse step's end point is gone: bisection for further surfaces
-                    search(p, st);
-                } else if (S::FP64 && sbest == s && evbest == ev) {
+                    const int e = __ffs(pending) - 1;
+                    search(p, st, e == 0 ? g1[0] : e == 1 ? g1[1] : e == 2 ? g1[2] : g1[3]);
+                } else if (S::FP64 && same(sbest, s) && evbest == ev) {
                     land = true;  // the last trial step ended on the crossing: no re-evaluation
                 } else {
                     phase = PH_FINAL;
@@ -1036,12 +1058,11 @@ struct Lane {
         }
         return status;
     }
-    // start the search for the next pending surface
-    __device__ __forceinline__ void search(const Params &p, const S &st) {
+    // start the search for the next pending surface; g: its event function at the end point of the step
+    __device__ __forceinline__ void search(const Params &p, const S &st, R g) {
         ev = __ffs(pending) - 1;
-        lo = 0; hi = hs; glo = st.g_start(p, ev);
-        ghi = ev == 0 ? g1[0] : ev == 1 ? g1[1] : ev == 2 ? g1[2] : g1[3];
-        if (!(glo <= (R)0)) glo = 0;
+        lo = 0; hi = hs; glo = st.g_start(p, ev); ghi = g;
+        if (!not_positive(glo)) glo = 0;
         side = 0; it = 0;
     }
 };

@@ -68,6 +68,7 @@ struct Params {
     // (0 without a band); R2^2 and H/2 as float-float for the event functions of the crossing search
     float R1f, R2f, halfHf, Kf, invKf, R1sq_hf, R1sq_lf, band_limf;
     float R2sq_hf, R2sq_lf, halfH_hf, halfH_lf;
+    double gtol_lat, gtol_cap, gtol_metal;  // |g| at which a point counts as on the surface
     int dedicated_blocks;  // batched integration: blocks whose warps take the reserved long rays
     // schedule knobs (results do not depend on them): blocks for the slowest rays, rays reserved for them
     // per thread, resolution of the cost buckets (bucket = cost_scale x -log2 |L_z|)
@@ -644,20 +645,18 @@ enum { EV_LAT = 0, EV_TOP = 1, EV_BOT = 2, EV_METAL = 3 };
 // which has the same roots and signs as r - R and needs no square root.
 // Rate of change of the event function along a motion dx of the position x: grad g(x) . dx.
 __device__ __forceinline__ double event_dg(int ev, const double x[3], const double dx[3]) {
-    switch (ev) {
-    case EV_LAT: return 2.0 * fma(x[0], dx[0], x[1] * dx[1]);
-    case EV_TOP: return dx[2];
-    case EV_BOT: return -dx[2];
-    default: return -2.0 * fma(x[0], dx[0], x[1] * dx[1]);
-    }
+    const double m = fma(x[0], dx[0], __dmul_rn(x[1], dx[1]));
+    const double r = ev == EV_LAT || ev == EV_METAL ? m + m : dx[2];
+    return ev == EV_BOT || ev == EV_METAL ? -r : r;
+}
+// rr: x^2 + y^2 (one FP64 operation for every surface: lanes of a warp that cross different ones do not diverge)
+__device__ __forceinline__ double event_g(const Params &p, int ev, double rr, double z) {
+    const double a = ev == EV_LAT ? rr : ev == EV_TOP ? z : ev == EV_BOT ? -z : p.R1sq;
+    const double b = ev == EV_LAT ? p.R2sq : ev == EV_METAL ? rr : p.halfH;
+    return a - b;
 }
 __device__ __forceinline__ double event_g(const Params &p, int ev, const double y[6]) {
-    switch (ev) {
-    case EV_LAT: return fma(y[0], y[0], y[1] * y[1]) - p.R2sq;
-    case EV_TOP: return y[2] - p.halfH;
-    case EV_BOT: return -y[2] - p.halfH;
-    default: return p.R1sq - fma(y[0], y[0], y[1] * y[1]);
-    }
+    return event_g(p, ev, fma(y[0], y[0], __dmul_rn(y[1], y[1])), y[2]);
 }
 
 // The crossing search (Lane, integrator.cuh): root s* in (0, h] of g(flow_s(y)) for a surface crossed by the step
@@ -676,9 +675,11 @@ constexpr double CROSS_REL_TOL = 1e-13;
 // Regula falsi also stops at a trial point where |g| <= CROSS_G_TOL times the surface's scale (R2^2,
 // R1^2 or H/2): the point lies on the surface to the rounding of g.
 constexpr double CROSS_G_TOL = 4e-16;
-__device__ __forceinline__ double cross_g_scale(const Params &p, int ev) {
-    return ev == EV_LAT ? p.R2sq : ev == EV_METAL ? p.R1sq : p.halfH;
+// (CROSS_G_TOL x R2^2, H/2, H/2, R1^2 for the four surfaces, rounded on the host)
+__device__ __forceinline__ double cross_g_tol(const Params &p, int ev) {
+    return ev == EV_LAT ? p.gtol_lat : ev == EV_METAL ? p.gtol_metal : p.gtol_cap;
 }
+
 // First entry of o + s d into the finite cylinder r <= R2, |z| <= H/2.
 // face: EV_LAT / EV_TOP / EV_BOT, or -1 for a miss.
 __device__ __forceinline__ int cylinder_entry(const Params &p, const double o[3], const double d[3], double pt[3],

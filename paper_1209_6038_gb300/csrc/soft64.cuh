@@ -140,6 +140,15 @@ S64_FN bool s64_positive(double a) {
     const int64_t b = s64_bits(a);
     return b > 0 && b <= 0x7ff0000000000000ll;
 }
+// a <= 0, a >= 0 for any a (false for NaN)
+S64_FN bool s64_not_positive(double a) {
+    const int64_t b = s64_bits(a);
+    return b == 0 || (b < 0 && (uint64_t)b <= 0xfff0000000000000ull);
+}
+S64_FN bool s64_not_negative(double a) {
+    const uint64_t b = (uint64_t)s64_bits(a);
+    return b <= 0x7ff0000000000000ull || b == 0x8000000000000000ull;
+}
 S64_FN double s64_abs(double a) {
     return s64_make((uint32_t)s64_hi(a) & 0x7fffffffu, (uint32_t)s64_lo(a));
 }

@@ -247,6 +247,9 @@ __device__ __noinline__ void wf_integrate_wide(const Params &kp, const Queue &q,
     p.R1sq = kp.R1sq;
     p.R2sq = kp.R2sq;
     p.halfH = kp.halfH;
+    p.gtol_lat = kp.gtol_lat;
+    p.gtol_cap = kp.gtol_cap;
+    p.gtol_metal = kp.gtol_metal;
     p.R1f = kp.R1f;
     p.h_or_tol = kp.h_or_tol;
     p.max_steps = kp.max_steps;
@@ -463,9 +466,13 @@ constexpr auto wf_integrate_kernel() {
     if constexpr (PREC != 1) return k_wf_integrate<VAR, MODE, INTEG, PREC>;
     else return k_wf_integrate_mixed<VAR, MODE, INTEG, PREC>;
 }
-// rays reserved for the long-ray blocks: reserve_per_thread for each ray that their warps advance at a time
-inline unsigned int long_ray_reserve(const Params &p, int prec, int packet) {
-    return (unsigned int)(p.long_ray_blocks * (prec == 0 ? packet / WIDE_LANES : packet) * p.reserve_per_thread);
+// Rays reserved for the long-ray blocks: reserve_per_thread for each of their threads; FP64 Fermat form, where a
+// ray takes eight: reserve_per_thread for each ray that they advance at a time, in a batch four times that
+// (twelve views 1920 x 1080 x 4: one 651, four 622, eight 622 ms; single images, whose bulk is done before the
+// slowest ray: 481 x 271 x 3 one 58.8, four 70.0, eight 96 ms, 1920 x 1080 x 4 one 188, four 209).
+inline unsigned int long_ray_reserve(const Params &p, int prec, int packet, bool batch) {
+    const int per_block = prec == 0 ? (batch ? 4 : 1) * (packet / WIDE_LANES) : packet;
+    return (unsigned int)(p.long_ray_blocks * per_block * p.reserve_per_thread);
 }
 // the kernel's precision index from the handle's settings
 inline int wf_prec(const Params &p) { return p.precision ? 1 : p.formulation ? 2 : 0; }
@@ -566,7 +573,7 @@ static cudaError_t wavefront_vmip(const Params &p, int spp, unsigned long long s
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int pk = packet > 0 ? packet : 128;
     // the slowest rays go to the warps of LONG_RAY_BLOCKS blocks that have their SMs to themselves
-    k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS, long_ray_reserve(p, PREC, pk));
+    k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS, long_ray_reserve(p, PREC, pk, false));
     k_wf_sort_scatter<<<sms * 8, 256, 0, st>>>(q);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
