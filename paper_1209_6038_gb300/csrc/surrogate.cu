@@ -208,6 +208,17 @@ __global__ void k_sur_unpack(const float *Y, long long n, float *y) {
 #pragma unroll
     for (int j = 0; j < SUR_OUT; ++j) y[i * SUR_OUT + j] = Y[(size_t)i * 16 + j];
 }
+// One layer's gradients in the C ABI's flat layout (W out x in, row-major, then b) at dst; the first layer's weight
+// gradient is the sum of its input's two columns (hi and lo parts).
+__global__ void k_sur_flat_grad(SurDims dm, const float *gW, const float *gb, float *dst) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x, nw = dm.out * dm.in;
+    if (e < nw) {
+        const size_t k = (size_t)(e / dm.in) * dm.kin + e % dm.in;
+        dst[e] = dm.in == SUR_IN ? gW[k] + gW[k + SUR_IN] : gW[k];
+    } else if (e < nw + dm.out) {
+        dst[e] = gb[e - nw];
+    }
+}
 // FP32 targets (n x 8) into the batch target buffer, and FP32 inputs into the batch input buffers
 __global__ void k_sur_pack_batch(const float *x, const float *t, int B, __nv_bfloat16 *Xb, __nv_bfloat16 *XTb,
                                  float *Tb) {
@@ -259,6 +270,7 @@ static bool tmap(CUtensorMap *m, const void *base, long long rows, int cols, int
     return make_tmap_bf16(m, base, (int)rows, cols, box_rows) == CUDA_SUCCESS;
 }
 
+static void drop_grad_ws(SurNet *s);
 SurNet *sur_create(double R1, double R2, double H, unsigned long long seed, const char **why) {
     SurNet *s = new SurNet();
     memset(s, 0, sizeof(*s));
@@ -345,6 +357,7 @@ void sur_destroy(SurNet *s) {
     if (!s) return;
     if (s->inf_arena) cudaFree(s->inf_arena);
     if (s->arena) cudaFree(s->arena);
+    drop_grad_ws(s);
     delete s;
 }
 
@@ -391,6 +404,8 @@ cudaError_t sur_forward(SurNet *s, long long n, const unsigned int *m_count, cud
 struct TrainWS {
     int B;
     char *arena;
+    size_t bytes;
+    float *flat;  // the gradient in the C ABI's layout (k_sur_flat_grad)
     __nv_bfloat16 *Xb, *XTb, *H[4], *HT[4], *dY, *dYT, *dZ[2], *dZT[2];
     float *Tb, *Z[4], *Y;
     double *loss;
@@ -412,7 +427,9 @@ static cudaError_t ws_create(TrainWS &w, int B, cudaStream_t st) {
     const size_t x = align256((size_t)B * 64 * 2), z = align256((size_t)B * SUR_W * 4),
                  h = align256((size_t)B * SUR_W * 2), t = align256((size_t)B * SUR_TSTRIDE * 4),
                  y = align256((size_t)B * 16 * 4), dyt = align256((size_t)128 * B * 2);
-    const size_t bytes = 2 * x + t + 4 * z + 8 * h + y + x + dyt + 4 * h + 512 + part;
+    const size_t flat = align256((size_t)sur_nparams() * 4);
+    const size_t bytes = 2 * x + t + 4 * z + 8 * h + y + x + dyt + 4 * h + 512 + part + flat;
+    w.bytes = bytes;
     cudaError_t e = cudaMalloc(&w.arena, bytes);
     if (e != cudaSuccess) return e;
     // cleared on the stream that uses it (a cudaMemset on the legacy default stream can still be running
@@ -433,6 +450,7 @@ static cudaError_t ws_create(TrainWS &w, int B, cudaStream_t st) {
     w.loss = (double *)p;
     w.sched = (SurSched *)(p + 256);
     w.partials = (float *)(p + 512);
+    w.flat = (float *)(p + 512 + part);
     bool ok = tmap(&w.tXb, w.Xb, B, 64, GEMM_TILE_M) && tmap(&w.tXTb, w.XTb, 64, B, 64) &&
               tmap(&w.tdY, w.dY, B, 64, GEMM_TILE_M) && tmap(&w.tdYT, w.dYT, 128, B, GEMM_TILE_M);
     for (int l = 0; l < 4; ++l)
@@ -444,6 +462,29 @@ static cudaError_t ws_create(TrainWS &w, int B, cudaStream_t st) {
 static void ws_destroy(TrainWS &w) {
     if (w.arena) cudaFree(w.arena);
     w.arena = nullptr;
+}
+// The workspace of a batch gradient stays with the network for the next batch of the same size, up to this many
+// bytes (allocating and clearing 130 MB took half of a call's time at the training batch); its padding, cleared
+// when it is made, is never written.
+constexpr size_t GRAD_WS_KEEP = (size_t)1 << 30;
+static cudaError_t grad_workspace(SurNet *s, int B, cudaStream_t st, TrainWS **out) {
+    if (s->grad_ws && s->grad_ws->B != B) drop_grad_ws(s);
+    if (!s->grad_ws) {
+        s->grad_ws = new TrainWS();
+        const cudaError_t e = ws_create(*s->grad_ws, B, st);
+        if (e != cudaSuccess) {
+            drop_grad_ws(s);
+            return e;
+        }
+    }
+    *out = s->grad_ws;
+    return cudaSuccess;
+}
+static void drop_grad_ws(SurNet *s) {
+    if (!s->grad_ws) return;
+    ws_destroy(*s->grad_ws);
+    delete s->grad_ws;
+    s->grad_ws = nullptr;
 }
 
 // split of the batch dimension for the weight-gradient GEMMs: about one CTA per SM
@@ -689,9 +730,10 @@ int sur_forward_rows(SurNet *s, const float *dev_x, long long n, float *dev_y, c
 // gradients (host, flat layout) of one batch, and optionally one Adam step with learning rate lr
 int sur_batch_grad(SurNet *s, const float *dev_x, const float *dev_t, long long n, int stage, double lr,
                    float *host_grad, cudaStream_t st, std::string &why) {
-    TrainWS w;
-    cudaError_t e = ws_create(w, (int)n, st);
-    if (e != cudaSuccess) { ws_destroy(w); why = "cannot allocate the training workspace"; return CLOAK_ENOMEM; }
+    TrainWS *kept = nullptr;
+    cudaError_t e = grad_workspace(s, (int)n, st, &kept);
+    if (e != cudaSuccess) { why = "cannot allocate the training workspace"; return CLOAK_ENOMEM; }
+    TrainWS &w = *kept;
     unsigned int *err = s->err;  // this network's own timeout flag
     cudaMemsetAsync(err, 0, 4, st);
     cudaMemsetAsync(w.loss, 0, 8, st);
@@ -711,24 +753,21 @@ int sur_batch_grad(SurNet *s, const float *dev_x, const float *dev_t, long long 
             e = train_backward(s, w, 0, st);
         }
     }
+    if (e == cudaSuccess && host_grad) {
+        long long o = 0;
+        for (int l = 0; l < SUR_L; ++l) {
+            const SurDims d = sur_dims(l);
+            const int m = d.out * d.in + d.out;
+            k_sur_flat_grad<<<(m + 255) / 256, 256, 0, st>>>(d, s->gW[l], s->gb[l], w.flat + o);
+            o += m;
+        }
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(host_grad, w.flat, (size_t)o * 4, cudaMemcpyDeviceToHost, st);
+    }
     unsigned int h = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, err, 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess && host_grad) {
-        std::vector<float> buf;
-        long long o = 0;
-        for (int l = 0; l < SUR_L && e == cudaSuccess; ++l) {
-            SurDims d = sur_dims(l);
-            buf.resize((size_t)d.mw * d.kin);
-            e = cudaMemcpy(buf.data(), s->gW[l], buf.size() * 4, cudaMemcpyDeviceToHost);
-            for (int r = 0; r < d.out; ++r)
-                for (int c = 0; c < d.in; ++c)
-                    host_grad[o++] = buf[(size_t)r * d.kin + c] + (l == 0 ? buf[(size_t)r * d.kin + SUR_IN + c] : 0.f);
-            if (e == cudaSuccess) e = cudaMemcpy(host_grad + o, s->gb[l], (size_t)d.out * 4, cudaMemcpyDeviceToHost);
-            o += d.out;
-        }
-    }
-    ws_destroy(w);
+    if (e != cudaSuccess || w.bytes > GRAD_WS_KEEP) drop_grad_ws(s);
     if (e != cudaSuccess) { why = cudaGetErrorString(e); return CLOAK_ECUDA; }
     if (h) { why = "tensor-core GEMM timed out"; return CLOAK_ETIMEOUT; }
     return CLOAK_OK;

@@ -52,6 +52,7 @@ __host__ __device__ inline SurDims sur_dims(int l) {
     return d;
 }
 
+struct TrainWS;
 struct SurNet {
     // parameters, FP32 master copies (W: mw x kin, zero outside out x in; b: mw)
     float *W[SUR_L], *b[SUR_L];
@@ -80,6 +81,8 @@ struct SurNet {
     int inf_f16;  // inference operands: 0 = BF16 (the training precision, default), 1 = FP16
     float *Y;
     unsigned char *elig;
+    // workspace of the last batch gradient, kept for the next of the same size (surrogate.cu)
+    TrainWS *grad_ws;
 };
 
 // lifetime and parameters (surrogate.cu)
