@@ -2,11 +2,11 @@
 //
 //   C[M x N] = A[M x K] * B[N x K]^T      A, B row-major BF16 (K contiguous), FP32 accumulation.
 //
-// One CTA (4 warps) computes a 128 x N tile (N <= 256, multiple of 16) over one slice of K (split-K:
+// One CTA (16 warps) computes a 128 x N tile (N <= 256, multiple of 16) over one slice of K (split-K:
 // gridDim.y slices).  K is consumed in chunks of 64 elements (128 bytes, one 128B-swizzle row): warp 0 /
 // lane 0 issues the TMA loads of A and B chunks into a 3-stage shared-memory ring and the tcgen05.mma
 // instructions (M = 128, K = 16 each, accumulator in tensor memory), committing each stage back to its
-// "empty" barrier.  After the last MMA completes, every warp reads its 32 accumulator lanes with
+// "empty" barrier.  After the last MMA completes, every warp reads its share of the accumulators with
 // tcgen05.ld and applies the epilogue (row r, column c, accumulator a):
 //   EPI_STORE     C[r, c] = a
 //   EPI_ATOMIC    C[r, c] += a                                (split-K partial sums, FP32 atomics)
@@ -50,6 +50,7 @@ struct GemmArgs {
 };
 
 constexpr int GEMM_TILE_M = 128;
+constexpr int GEMM_THREADS = 512;
 constexpr int GEMM_KCHUNK = 64;
 constexpr int GEMM_STAGES = 2;  // K of the network's layers is at most 256: four chunks, double-buffered
 
