@@ -7,11 +7,14 @@
 //     128-byte swizzle) through a 3-slot ring, refilling a slot as soon as the MMAs that read it are done,
 //     and loads each tile's inputs (the K-major layout the MMA reads) once the tile's previous last-layer
 //     MMAs are done -- after the weight chunk of the tile's first job, so that chunk is already on its way;
-//   * the MMA warp (one thread) issues, per chunk, the four tcgen05.mma (M = 128, K = 16) of the job's tile
+//   * the MMA warp (the whole warp in step, one elected lane issuing) issues, per chunk, the four tcgen05.mma (M = 128, K = 16) of the job's tile
 //     (one for the first layer, whose 14 input columns fit one K step) into its TMEM columns (tile t:
 //     256 t .. 256 t + 255) and frees the slot by a commit.  Before a job's
 //     first MMA it waits only for the epilogue of the same tile's previous layer, so the MMAs of one tile
-//     run while the epilogue of the other tile runs.  The two roles are separate threads because one
+//     run while the epilogue of the other tile runs.  In a branch of one thread the compiler cannot keep the
+//     descriptors and barrier addresses in uniform registers and replays each instruction per active lane: with the
+//     warp in step 1,000,003 rows take 605 us instead of 668 (BF16), and a bare stream of these MMAs with its
+//     waits 1.08 ms instead of 1.20.  The two roles are separate threads because one
 //     thread doing both spent longer per chunk on its barrier waits and bookkeeping than the tensor core
 //     spent on the chunk's four MMAs;
 //   * 16 epilogue warps take the jobs in the same order (warp w: TMEM lanes 32 (w % 4) .., column quarter
@@ -169,30 +172,32 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                 if (x_pending[t]) mbar_wait(smem_u32(&x_bar[t]), x_phase[t]);
         }
     } else if (warp == F_MMA_WARP) {
-        if (lane == 0) {
-            uint32_t s = 0, ph = 0;  // ring slot of the next chunk and its fill parity
-            uint32_t Lt[2] = {0, 0}; // jobs committed per tile (phases of done_bar[t] / act_bar[t])
-            uint32_t iters = 0;      // tile pairs started (phase of x_bar[t])
-            bool ok = true;
-            const uint32_t ring0 = smem_u32(ring), act0 = smem_u32(act);
-            for (long long base = (long long)blockIdx.x * 256; base < live && ok; base += stride) {
-                for (int job = 0; job < 2 * SUR_L && ok; ++job) {
-                    const int l = job >> 1, t = job & 1;
-                    const int nk = l == 0 ? 1 : 4;
-                    const uint32_t idesc = F16 ? f16_idesc(l == SUR_L - 1 ? 16 : SUR_W) : bf16_idesc(l == SUR_L - 1 ? 16 : SUR_W);
-                    const uint32_t d_tmem = tmem + t * 256;
-                    for (int j = 0; j < nk; ++j) {
-                        ok = mbar_wait(smem_u32(&full_bar[s]), ph, lim);
-                        if (ok && j == 0) {
-                            // the tile's previous epilogue has read its accumulators and written these inputs
-                            if (Lt[t] > 0) ok = mbar_wait(smem_u32(&act_bar[t]), (Lt[t] - 1) & 1, lim);
-                            if (ok && l == 0) ok = mbar_wait(smem_u32(&x_bar[t]), iters & 1, lim);
-                            if (ok && *vfailed) ok = false;
-                        }
-                        if (!ok) break;
-                        asm volatile("tcgen05.fence::after_thread_sync;");
-                        const uint64_t bd = sw128_desc(ring0 + s * F_RING_SLOT);
-                        const uint64_t ad = sw128_desc(act0 + (uint32_t)(t * 4 + j) * F_ACT_CHUNK);
+        // the whole warp walks the jobs and waits; one elected lane issues
+        uint32_t s = 0, ph = 0;  // ring slot of the next chunk and its fill parity
+        uint32_t Lt[2] = {0, 0}; // jobs committed per tile (phases of done_bar[t] / act_bar[t])
+        uint32_t iters = 0;      // tile pairs started (phase of x_bar[t])
+        bool ok = true;
+        const uint32_t ring0 = smem_u32(ring), act0 = smem_u32(act);
+        for (long long base = (long long)blockIdx.x * 256; base < live && ok; base += stride) {
+            for (int job = 0; job < 2 * SUR_L && ok; ++job) {
+                const int l = job >> 1, t = job & 1;
+                const int nk = l == 0 ? 1 : 4;
+                const uint32_t idesc = F16 ? f16_idesc(l == SUR_L - 1 ? 16 : SUR_W) : bf16_idesc(l == SUR_L - 1 ? 16 : SUR_W);
+                const uint32_t d_tmem = tmem + t * 256;
+                for (int j = 0; j < nk; ++j) {
+                    ok = mbar_wait(smem_u32(&full_bar[s]), ph, lim);
+                    if (ok && j == 0) {
+                        // the tile's previous epilogue has read its accumulators and written these inputs
+                        if (Lt[t] > 0) ok = mbar_wait(smem_u32(&act_bar[t]), (Lt[t] - 1) & 1, lim);
+                        if (ok && l == 0) ok = mbar_wait(smem_u32(&x_bar[t]), iters & 1, lim);
+                        if (ok && *vfailed) ok = false;
+                    }
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint64_t bd = sw128_desc(ring0 + s * F_RING_SLOT);
+                    const uint64_t ad = sw128_desc(act0 + (uint32_t)(t * 4 + j) * F_ACT_CHUNK);
+                    if (elect_one()) {
                         // the first layer's inputs (7 values as hi/lo pairs) and weights fill K columns 0..13 of
                         // the chunk and are zero beyond: one MMA covers them
                         const int nmma = l == 0 ? 1 : 4;
@@ -207,24 +212,25 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                         }
                         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                             smem_u32(&empty_bar[s])));
-                        if (++s == F_SLOTS) { s = 0; ph ^= 1u; }
+                        if (j == nk - 1)
+                            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                smem_u32(&done_bar[t])));
                     }
-                    if (!ok) break;
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                        smem_u32(&done_bar[t])));
-                    ++Lt[t];
+                    __syncwarp();
+                    if (++s == F_SLOTS) { s = 0; ph ^= 1u; }
                 }
-                ++iters;
+                ++Lt[t];
             }
-            if (!ok) {
-                *vfailed = 1;
-                if (a.err) atomicExch(a.err, 1u);
-                // the MMAs already issued complete before the accumulators are freed (a commit arrives once every
-                // earlier MMA of this thread is done); bounded by the default limit
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                    smem_u32(&drain_bar)));
-                mbar_wait(smem_u32(&drain_bar), 0);
-            }
+            ++iters;
+        }
+        if (!ok && elect_one()) {
+            *vfailed = 1;
+            if (a.err) atomicExch(a.err, 1u);
+            // the MMAs already issued complete before the accumulators are freed (a commit arrives once every
+            // earlier MMA of this thread is done); bounded by the default limit
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                smem_u32(&drain_bar)));
+            mbar_wait(smem_u32(&drain_bar), 0);
         }
     } else {
         // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (one row per thread), column quarter w / 4
