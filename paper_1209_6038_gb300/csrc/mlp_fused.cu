@@ -27,11 +27,18 @@
 // in, or -- selected per network -- FP16: the GELU is evaluated in half-precision pairs in both forms, and
 // in FP16 its result is stored as it is (no conversion back through FP32 to BF16: faster, and 11
 // significant bits instead of 8).  Accumulation is FP32 in both.
+// The public forward call's FP32 rows come in through one more warp, which splits them into the pairs and writes
+// them where the TMA load of packed rows would (the next pair's rows are in registers before the tile is free), and
+// its outputs go straight to the caller's rows: packing to 128-byte rows and unpacking from 64-byte ones moved 340
+// bytes a row in two more launches, and the copy warp's wait for a free tile held up the weights behind it.
+// 1,000,003 rows 605 -> 457 us, bit for bit the same.  Bound now by the
+// epilogue and its hand-over to the MMAs: tensor pipe about a third busy.
 // Barriers: full/empty per ring slot; per tile the inputs' barrier, "MMAs done" (committed by the MMA
-// warp) and "activations ready" (16 arrivals).  Shared memory: activations 2 x 64 KB, weight ring
+// warp), "activations free" (its last layer's) and "activations ready" (16 arrivals).  Shared memory: activations 2 x 64 KB, weight ring
 // 3 x 32 KB.  Every mbarrier wait is bounded; on a timeout the kernel sets the error flag, lets its MMAs and
 // copies in flight complete, frees TMEM and returns.
 #include "device_once.h"
+#include "sur_physics.cuh"
 #include "surrogate.h"
 #include "tc_ptx.cuh"
 
@@ -41,7 +48,8 @@ namespace {
 constexpr int F_EPI_WARPS = 16;
 constexpr int F_COPY_WARP = F_EPI_WARPS;                       // warp index of the TMA copy thread
 constexpr int F_MMA_WARP = F_EPI_WARPS + 1;                    // warp index of the MMA thread
-constexpr int F_THREADS = 32 * (F_EPI_WARPS + 2);
+constexpr int F_IN_WARP = F_EPI_WARPS + 2;                     // warp index of the input rows (FP32 rows only)
+constexpr int F_THREADS = 32 * (F_EPI_WARPS + 3);
 constexpr int F_PARTS = F_EPI_WARPS / 4;                       // epilogue warps per row quarter (column parts)
 constexpr uint32_t F_ACT_CHUNK = 128 * 128;                  // 128 rows x 64 BF16 = 16 KB
 constexpr uint32_t F_ACT_BYTES = 2 * 4 * F_ACT_CHUNK;         // 2 tiles x 4 K chunks
@@ -52,8 +60,9 @@ constexpr size_t F_SMEM = 1024 + F_ACT_BYTES + F_SLOTS * F_RING_SLOT;
 struct FusedArgs {
     const float *bias[SUR_L];    // FP32 biases (the output layer's are used)
     const __half *bias_h[SUR_L - 1]; // hidden layers' biases in half precision (both forms)
-    float *Y;                    // outputs, 16 FP32 per row
-    long long n;                 // rows of X and Y (a multiple of 128)
+    const float *x;              // FP32 input rows (SUR_IN each); null: the packed rows behind the tensor map
+    float *Y;                    // outputs: SUR_OUT FP32 per row with x, else 16
+    long long n;                 // rows of x / X and Y
     const unsigned int *m_count; // optional live row count
     unsigned int *err;
     unsigned int wait_limit;     // polls of the waits that decide a timeout
@@ -85,12 +94,12 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                 const __grid_constant__ CUtensorMap tW1, const __grid_constant__ CUtensorMap tW2,
                 const __grid_constant__ CUtensorMap tW3, const __grid_constant__ CUtensorMap tW4, FusedArgs a) {
     extern __shared__ unsigned char fsm_raw[];
-    __shared__ __align__(8) uint64_t full_bar[F_SLOTS], empty_bar[F_SLOTS], x_bar[2], done_bar[2], act_bar[2], drain_bar;
+    __shared__ __align__(8) uint64_t full_bar[F_SLOTS], empty_bar[F_SLOTS], x_bar[2], done_bar[2], act_bar[2], free_bar[2], drain_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
     unsigned char *sm = (unsigned char *)(((uintptr_t)fsm_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *act = sm, *ring = sm + F_ACT_BYTES;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const long long live = a.m_count ? min(a.n, (long long)__ldg(a.m_count)) : a.n;
     volatile int *vfailed = &failed;
     const uint32_t lim = a.wait_limit;
@@ -104,6 +113,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
             mbar_init(smem_u32(&x_bar[t]), 1);
             mbar_init(smem_u32(&done_bar[t]), 1);
             mbar_init(smem_u32(&act_bar[t]), F_EPI_WARPS);
+            mbar_init(smem_u32(&free_bar[t]), 1);
         }
         mbar_init(smem_u32(&drain_bar), 1);
         failed = 0;
@@ -144,7 +154,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                         if (++s == F_SLOTS) { s = 0; ph ^= 1u; }
                     }
                     if (!ok) break;
-                    if (l == 0) {
+                    if (l == 0 && !a.x) {
                         // the tile's inputs overwrite its activations, which its previous last-layer MMAs read
                         // ("MMAs done" completes SUR_L times per tile and pair)
                         if (Lx > 0) ok = mbar_wait(smem_u32(&done_bar[t]), (SUR_L * Lx - 1) & 1, lim);
@@ -215,6 +225,9 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                         if (j == nk - 1)
                             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                 smem_u32(&done_bar[t])));
+                        if (l == SUR_L - 1 && j == nk - 1)
+                            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                smem_u32(&free_bar[t])));
                     }
                     __syncwarp();
                     if (++s == F_SLOTS) { s = 0; ph ^= 1u; }
@@ -231,6 +244,46 @@ __global__ void __launch_bounds__(F_THREADS, 1)
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                 smem_u32(&drain_bar)));
             mbar_wait(smem_u32(&drain_bar), 0);
+        }
+    } else if (warp == F_IN_WARP) {
+        // FP32 rows: split into the first layer's (hi, lo) pairs in the swizzled layout, four rows of a tile per lane,
+        // loaded before the tile's activations are free to be overwritten
+        bool ok = true;
+        uint32_t Lx = 0;
+        for (long long base = (long long)blockIdx.x * 256; a.x && base < live && ok; base += stride) {
+            for (int t = 0; t < 2; ++t) {
+                float x[4][SUR_IN];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const long long row = base + 128 * t + 32 * i + lane;
+#pragma unroll
+                    for (int j = 0; j < SUR_IN; ++j) x[i][j] = row < live ? __ldg(a.x + row * SUR_IN + j) : 0.f;
+                }
+                // the tile's previous last layer has read them (its own barrier: "MMAs done" completes SUR_L times per
+                // pair, and this warp is early enough to take an earlier layer's phase for the last one's)
+                if (Lx > 0) ok = mbar_wait(smem_u32(&free_bar[t]), (Lx - 1) & 1, lim);
+                ok = __all_sync(0xffffffffu, ok && !*vfailed);
+                if (!ok) break;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = 32 * i + lane;
+                    __align__(16) uint16_t v[16];
+                    v[14] = v[15] = 0;
+#pragma unroll
+                    for (int j = 0; j < SUR_IN; ++j) sur_split_pair(x[i][j], F16, v + j, v + SUR_IN + j);
+                    unsigned char *dst = act + t * 4 * F_ACT_CHUNK + (r >> 3) * 1024 + (r & 7) * 128;
+                    *(uint4 *)(dst + ((r & 7) << 4)) = *(const uint4 *)v;
+                    *(uint4 *)(dst + ((1 ^ (r & 7)) << 4)) = *(const uint4 *)(v + 8);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&x_bar[t]));
+            }
+            ++Lx;
+        }
+        if (!ok && lane == 0) {
+            *vfailed = 1;
+            if (a.err) atomicExch(a.err, 1u);
         }
     } else {
         // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (one row per thread), column quarter w / 4
@@ -274,7 +327,11 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                     tmem_ld16(taddr, u);
                     tmem_wait16(u);
                     const long long row = base + t * 128 + r;
-                    if (row < live) {
+                    if (row < live && a.x) {
+                        float *y = a.Y + row * SUR_OUT;
+#pragma unroll
+                        for (int i = 0; i < SUR_OUT; ++i) y[i] = __uint_as_float(u[i]) + __ldg(a.bias[SUR_L - 1] + i);
+                    } else if (row < live) {
                         float4 *y = (float4 *)(a.Y + row * 16);
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
@@ -325,34 +382,45 @@ cudaError_t mlp_fused_prepare() {
     });
 }
 
-// forward pass of rows [0, n) of s->X into s->Y (rows beyond *m_count skipped when it is set)
-cudaError_t launch_mlp_fused(SurNet *s, long long n, const unsigned int *m_count, cudaStream_t st) {
-    cudaError_t e0 = mlp_fused_prepare();
-    if (e0 != cudaSuccess) return e0;
+static cudaError_t launch(SurNet *s, const CUtensorMap &tx, const float *x, float *y, long long n,
+                          const unsigned int *m_count, cudaStream_t st) {
     int dev = 0;
     cudaGetDevice(&dev);
-    const int sms = g_fused_sms[dev];
-    if (n <= 0 || n % 128) return cudaErrorInvalidValue;
-    CUtensorMap tx;
-    const bool f16 = s->inf_f16 != 0;
-    if ((f16 ? make_tmap_f16(&tx, s->X, (int)n, 64, GEMM_TILE_M) : make_tmap_bf16(&tx, s->X, (int)n, 64, GEMM_TILE_M)) !=
-        CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
     FusedArgs a;
     for (int l = 0; l < SUR_L; ++l) a.bias[l] = s->b[l];
     for (int l = 0; l < SUR_L - 1; ++l) a.bias_h[l] = s->bh[l];
-    a.Y = s->Y;
+    a.x = x;
+    a.Y = y;
     a.n = n;
     a.m_count = m_count;
     a.err = s->err;
     a.wait_limit = wait_limit();
     const long long pairs = (n + 255) / 256;
-    const int grid = (int)std::min<long long>(pairs, (long long)sms);
-    if (f16)
+    const int grid = (int)std::min<long long>(pairs, (long long)g_fused_sms[dev]);
+    if (s->inf_f16)
         k_mlp_fused<true><<<grid, F_THREADS, F_SMEM, st>>>(tx, s->tWh[0], s->tWh[1], s->tWh[2], s->tWh[3], s->tWh[4], a);
     else
         k_mlp_fused<false><<<grid, F_THREADS, F_SMEM, st>>>(tx, s->tWb[0], s->tWb[1], s->tWb[2], s->tWb[3], s->tWb[4], a);
     return cudaGetLastError();
+}
+
+// forward pass of rows [0, n) of s->X into s->Y (rows beyond *m_count skipped when it is set)
+cudaError_t launch_mlp_fused(SurNet *s, long long n, const unsigned int *m_count, cudaStream_t st) {
+    cudaError_t e = mlp_fused_prepare();
+    if (e != cudaSuccess) return e;
+    if (n <= 0 || n % 128) return cudaErrorInvalidValue;
+    CUtensorMap tx;
+    if ((s->inf_f16 ? make_tmap_f16(&tx, s->X, (int)n, 64, GEMM_TILE_M)
+                    : make_tmap_bf16(&tx, s->X, (int)n, 64, GEMM_TILE_M)) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return launch(s, tx, nullptr, s->Y, n, m_count, st);
+}
+
+// forward pass of n FP32 rows x (SUR_IN each) into y (SUR_OUT each), which do not overlap
+cudaError_t launch_mlp_fused_rows(SurNet *s, const float *x, float *y, long long n, cudaStream_t st) {
+    cudaError_t e = mlp_fused_prepare();
+    if (e != cudaSuccess) return e;
+    return launch(s, s->tWb[0], x, y, n, nullptr, st);  // the input map is not used
 }
 
 }  // namespace ck

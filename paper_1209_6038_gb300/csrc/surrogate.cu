@@ -732,16 +732,21 @@ cudaError_t sur_set_params(SurNet *s, const float *host) {
     return e;
 }
 
-// forward pass of n FP32 input rows (n x 7) into FP32 outputs (n x 5)
+// forward pass of n FP32 input rows (n x 7) into FP32 outputs (n x 5): the fused kernel reads and writes the rows
+// itself.  Only where outputs overlap the inputs they go through the padded scratch, which is filled before any
+// output is written.
 int sur_forward_rows(SurNet *s, const float *dev_x, long long n, float *dev_y, cudaStream_t st, std::string &why) {
-    cudaError_t e = sur_ensure_inference(s, n);
+    const bool overlap = (uintptr_t)dev_x < (uintptr_t)(dev_y + n * SUR_OUT) &&
+                         (uintptr_t)dev_y < (uintptr_t)(dev_x + n * SUR_IN);
+    cudaError_t e = overlap ? sur_ensure_inference(s, n) : cudaSuccess;
     if (e != cudaSuccess) { why = "cannot allocate the inference scratch"; return CLOAK_ENOMEM; }
     const long long rows = (n + 127) / 128 * 128;
     unsigned int *err = s->err;  // this network's own timeout flag
     cudaMemsetAsync(err, 0, 4, st);
-    k_sur_pack<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(dev_x, n, s->X, s->inf_f16);
-    if ((e = sur_forward(s, rows, nullptr, st)) != cudaSuccess) { why = cudaGetErrorString(e); return CLOAK_ECUDA; }
-    k_sur_unpack<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s->Y, n, dev_y);
+    if (overlap) k_sur_pack<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(dev_x, n, s->X, s->inf_f16);
+    e = overlap ? sur_forward(s, rows, nullptr, st) : launch_mlp_fused_rows(s, dev_x, dev_y, n, st);
+    if (e != cudaSuccess) { why = cudaGetErrorString(e); return CLOAK_ECUDA; }
+    if (overlap) k_sur_unpack<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s->Y, n, dev_y);
     unsigned int h = 0;
     cudaMemcpyAsync(&h, err, 4, cudaMemcpyDeviceToHost, st);
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) { why = cudaGetErrorString(e); return CLOAK_ECUDA; }

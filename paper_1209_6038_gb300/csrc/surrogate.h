@@ -94,6 +94,8 @@ cudaError_t sur_refresh_bf16(SurNet *s, cudaStream_t st);  // Wb / WTb / Wh / bh
 cudaError_t sur_forward(SurNet *s, long long n, const unsigned int *m_count, cudaStream_t st);
 // the same as one persistent tcgen05 kernel (mlp_fused.cu)
 cudaError_t launch_mlp_fused(SurNet *s, long long n, const unsigned int *m_count, cudaStream_t st);
+// the same from n FP32 rows x (n x 7) straight into y (n x 5), which must not overlap
+cudaError_t launch_mlp_fused_rows(SurNet *s, const float *x, float *y, long long n, cudaStream_t st);
 cudaError_t mlp_fused_prepare();  // one-time setup on the current device (call before capturing a forward pass)
 cudaError_t sur_ensure_inference(SurNet *s, long long rows);
 
