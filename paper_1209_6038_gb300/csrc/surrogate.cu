@@ -4,9 +4,9 @@
 // Training step on a batch of B rays (B a multiple of 128), every GEMM on the tensor cores (mlp_tc.cuh):
 //   forward  Z_l = H_{l-1} W_l^T + b_l, H_l = GELU(Z_l)          (H_{-1} = X; the last layer is affine)
 //   loss     dY = dL/dY                                           (k_sur_loss)
-//   backward dW_l = dZ_l^T H_{l-1}   (split over the batch, FP32 atomics)
+//   backward dW_l = dZ_l^T H_{l-1}   (split over the batch, slices summed in order)
 //            dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1})                (fused into the GEMM epilogue)
-//            db_l = column sums of dZ_l                            (k_sur_rowsum on the transposed copy)
+//            db_l = column sums of dZ_l                            (k_sur_reduce on the transposed copy)
 //   update   Adam on the FP32 masters, then their BF16 copies W_l and W_l^T (k_sur_adam)
 #include <algorithm>
 #include <atomic>
@@ -120,33 +120,51 @@ __global__ void k_sur_loss(const float *Y, const float *Tb, int B, int stage, __
     if ((threadIdx.x & 31) == 0 && L != 0.0) atomicAdd(loss, L);
 }
 
-// out[i] = sum over the slices s = 0, 1, ... of part[s * n + i], in that order: the weight gradients of the
-// batch-split GEMMs, summed the same way on every run (atomic accumulation made training order-dependent).
-// Bound by the latency of its loads: eight slices in flight per thread (76 slices of 256 x 256 11.0 -> 9.0 us).
-__global__ void k_sum_slices(const float *part, int slices, long long n, float *out) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        float acc = 0.f;
-        int k = 0;
-        for (; k + 8 <= slices; k += 8) {
-            float v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = part[(size_t)(k + j) * n + i];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc += v[j];
+// Gradients of one layer from what its GEMM left, in one launch.
+// Blocks below wblocks: gW[i] = sum over the slices of part[s * stride + i], i < n (multiples of 4), the batch-split weight
+// gradient, summed the same way on every run (atomic accumulation made training order-dependent): four outputs per
+// load, eight threads per output take a run of slices each and are added in order.  Bound by the latency of a
+// thread's loads: 76 slices of 256 x 256 took 9.0 us with one thread per output and 4.6 more for the bias, both 8.4 here
+// (11.0 and 38 at first); the output layer sums its 5 rows of 128 only.  A gradient of 19456 rows 390 -> 354 us.
+// The others: gb[r] = sum over the columns of row r of the transposed dZ, sixteen bytes per load (cols is a multiple
+// of 128, so rows are aligned); 19456 columns with one value per load took 38 us, 5 in a launch of its own.
+constexpr int RED_THREADS = 512, RED_PARTS = 8, RED_OUT = 4 * RED_THREADS / RED_PARTS;
+__global__ void __launch_bounds__(RED_THREADS) k_sur_reduce(const float *part, int slices, int n, int stride, float *gW,
+                                                            int wblocks, const __nv_bfloat16 *dZT, int cols, float *gb) {
+    if ((int)blockIdx.x < wblocks) {
+        constexpr int PER = RED_THREADS / RED_PARTS;
+        const int o = threadIdx.x % PER, g = threadIdx.x / PER, i = blockIdx.x * RED_OUT + 4 * o;
+        const int run = (slices + RED_PARTS - 1) / RED_PARTS, k1 = min(slices, (g + 1) * run);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < n) {
+#pragma unroll 10
+            for (int k = g * run; k < k1; ++k) {
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(part + (size_t)k * stride + i));
+                acc.x += v.x;
+                acc.y += v.y;
+                acc.z += v.z;
+                acc.w += v.w;
+            }
         }
-        for (; k < slices; ++k) acc += part[(size_t)k * n + i];
-        out[i] = acc;
+        __shared__ float4 sums[RED_PARTS][PER];
+        sums[g][o] = acc;
+        __syncthreads();
+        if (g == 0 && i < n) {
+            for (int k = 1; k < RED_PARTS; ++k) {
+                const float4 v = sums[k][o];
+                acc.x += v.x;
+                acc.y += v.y;
+                acc.z += v.z;
+                acc.w += v.w;
+            }
+            *reinterpret_cast<float4 *>(gW + i) = acc;
+        }
+        return;
     }
-}
-
-// out[r] = sum over the columns of row r of a BF16 matrix (bias gradients from a transposed dZ), a block per row.
-// Sixteen bytes per load (cols is a multiple of 128, so rows are aligned) and enough threads that a row is a few
-// loads deep: 19456 columns with one value per load took 38 us, 5 now.
-constexpr int ROWSUM_THREADS = 512;
-__global__ void __launch_bounds__(ROWSUM_THREADS) k_sur_rowsum(const __nv_bfloat16 *M, int cols, float *out) {
-    const uint4 *row = reinterpret_cast<const uint4 *>(M + (size_t)blockIdx.x * cols);
+    const int r = blockIdx.x - wblocks;
+    const uint4 *row = reinterpret_cast<const uint4 *>(dZT + (size_t)r * cols);
     float s = 0.f;
-    for (int c = threadIdx.x; c < cols / 8; c += ROWSUM_THREADS) {
+    for (int c = threadIdx.x; c < cols / 8; c += RED_THREADS) {
         const uint4 v = __ldg(row + c);
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
         float p = 0.f;
@@ -157,14 +175,14 @@ __global__ void __launch_bounds__(ROWSUM_THREADS) k_sur_rowsum(const __nv_bfloat
         }
         s += p;
     }
-    __shared__ float part[ROWSUM_THREADS / 32];
+    __shared__ float part_row[RED_THREADS / 32];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    if ((threadIdx.x & 31) == 0) part_row[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x < 32) {
-        s = threadIdx.x < ROWSUM_THREADS / 32 ? part[threadIdx.x] : 0.f;
+        s = threadIdx.x < RED_THREADS / 32 ? part_row[threadIdx.x] : 0.f;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) out[blockIdx.x] = s;
+        if (threadIdx.x == 0) gb[r] = s;
     }
 }
 
@@ -230,9 +248,15 @@ __global__ void k_sur_unpack(const float *Y, long long n, float *y) {
 #pragma unroll
     for (int j = 0; j < SUR_OUT; ++j) y[i * SUR_OUT + j] = Y[(size_t)i * 16 + j];
 }
-// One layer's gradients in the C ABI's flat layout (W out x in, row-major, then b) at dst; the first layer's weight
-// gradient is the sum of its input's two columns (hi and lo parts).
-__global__ void k_sur_flat_grad(SurDims dm, const float *gW, const float *gb, float *dst) {
+// The gradients in the C ABI's flat layout (per layer W out x in, row-major, then b) at dst, a layer per blockIdx.y;
+// the first layer's weight gradient is the sum of its input's two columns (hi and lo parts).
+struct SurGrads {
+    const float *gW[SUR_L], *gb[SUR_L];
+};
+__global__ void k_sur_flat_grad(SurGrads a, float *dst) {
+    const SurDims dm = sur_dims(blockIdx.y);
+    for (int l = 0; l < (int)blockIdx.y; ++l) dst += sur_dims(l).out * sur_dims(l).in + sur_dims(l).out;
+    const float *gW = a.gW[blockIdx.y], *gb = a.gb[blockIdx.y];
     const int e = blockIdx.x * blockDim.x + threadIdx.x, nw = dm.out * dm.in;
     if (e < nw) {
         const size_t k = (size_t)(e / dm.in) * dm.kin + e % dm.in;
@@ -432,7 +456,7 @@ struct TrainWS {
     float *Tb, *Z[4], *Y;
     double *loss;
     SurSched *sched;
-    float *partials;  // per-slice partial weight gradients (k_sum_slices)
+    float *partials;  // per-slice partial weight gradients (k_sur_reduce)
     CUtensorMap tXb, tXTb, tH[4], tHT[4], tdY, tdYT, tdZ[2], tdZT[2];
 };
 
@@ -540,19 +564,22 @@ static cudaError_t train_forward(SurNet *s, TrainWS &w, cudaStream_t st) {
     return e;
 }
 
-// dW = dZ^T H over the batch: the batch is split into K slices (about one CTA per SM), each slice stores
-// its partial product, and the slices are summed in a fixed order
-static cudaError_t weight_grad(SurNet *s, TrainWS &w, const SurDims &d, const CUtensorMap &tdz, const CUtensorMap &th,
-                               float *gW, cudaStream_t st) {
+// dW = dZ^T H over the batch and db, its column sums: the batch is split into K slices (about one CTA per SM), each
+// slice stores its partial product, and the slices are summed in a fixed order with the rows of dZ^T
+static cudaError_t layer_grad(SurNet *s, TrainWS &w, int l, const CUtensorMap &tdz, const CUtensorMap &th,
+                              const __nv_bfloat16 *dZT, cudaStream_t st) {
+    const SurDims d = sur_dims(l);
     GemmArgs g = gemm_args(d.mw, d.kin, w.B, EPI_STORE, s->err);
     g.ksplit = ksplit_for(w.B, d.mw / GEMM_TILE_M);
+    // the slices follow each other in full rows, of which the first d.out carry the layer
     g.C = w.partials;
     g.ldc = d.kin;
     g.slice_stride = (long long)d.mw * d.kin;
     cudaError_t e = gemm(tdz, th, g, st);
     if (e != cudaSuccess) return e;
-    const long long n = (long long)d.mw * d.kin;
-    k_sum_slices<<<(unsigned)std::min<long long>((n + 255) / 256, 1184), 256, 0, st>>>(w.partials, g.ksplit, n, gW);
+    const int n = d.out * d.kin, wblocks = (n + RED_OUT - 1) / RED_OUT;
+    k_sur_reduce<<<wblocks + d.out, RED_THREADS, 0, st>>>(w.partials, g.ksplit, n, (int)g.slice_stride, s->gW[l], wblocks,
+                                                         dZT, w.B, s->gb[l]);
     return cudaGetLastError();
 }
 
@@ -561,15 +588,11 @@ static cudaError_t train_backward(SurNet *s, TrainWS &w, int first, cudaStream_t
     cudaError_t e = cudaMemsetAsync(s->grad_begin, 0, s->grad_bytes, st);
     const int B = w.B;
     // output layer
-    {
-        SurDims d = sur_dims(SUR_L - 1);
-        if (e == cudaSuccess) e = weight_grad(s, w, d, w.tdYT, w.tHT[SUR_L - 2], s->gW[SUR_L - 1], st);
-        k_sur_rowsum<<<d.out, ROWSUM_THREADS, 0, st>>>(w.dYT, B, s->gb[SUR_L - 1]);
-    }
+    if (e == cudaSuccess) e = layer_grad(s, w, SUR_L - 1, w.tdYT, w.tHT[SUR_L - 2], w.dYT, st);
     int cur = 0;
     for (int l = SUR_L - 1; l > first && e == cudaSuccess; --l) {
         // dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1})
-        SurDims d = sur_dims(l), dp = sur_dims(l - 1);
+        SurDims d = sur_dims(l);
         const CUtensorMap &ta = l == SUR_L - 1 ? w.tdY : w.tdZ[cur ^ 1];
         GemmArgs g = gemm_args(B, d.kin, d.kb, EPI_GELU_BWD, s->err);
         g.Z = w.Z[l - 1]; g.ldz = SUR_W;
@@ -579,8 +602,7 @@ static cudaError_t train_backward(SurNet *s, TrainWS &w, int first, cudaStream_t
         if (e != cudaSuccess) break;
         // dW_{l-1} = dZ_{l-1}^T H_{l-2}, db_{l-1} = column sums of dZ_{l-1}
         const CUtensorMap &tb = l - 1 == 0 ? w.tXTb : w.tHT[l - 2];
-        e = weight_grad(s, w, dp, w.tdZT[cur], tb, s->gW[l - 1], st);
-        k_sur_rowsum<<<dp.out, ROWSUM_THREADS, 0, st>>>(w.dZT[cur], B, s->gb[l - 1]);
+        e = layer_grad(s, w, l - 1, w.tdZT[cur], tb, w.dZT[cur], st);
         cur ^= 1;
     }
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -781,15 +803,16 @@ int sur_batch_grad(SurNet *s, const float *dev_x, const float *dev_t, long long 
         }
     }
     if (e == cudaSuccess && host_grad) {
-        long long o = 0;
+        SurGrads a;
+        int m = 0;
         for (int l = 0; l < SUR_L; ++l) {
-            const SurDims d = sur_dims(l);
-            const int m = d.out * d.in + d.out;
-            k_sur_flat_grad<<<(m + 255) / 256, 256, 0, st>>>(d, s->gW[l], s->gb[l], w.flat + o);
-            o += m;
+            a.gW[l] = s->gW[l];
+            a.gb[l] = s->gb[l];
+            m = std::max(m, sur_dims(l).out * (sur_dims(l).in + 1));
         }
+        k_sur_flat_grad<<<dim3((m + 255) / 256, SUR_L), 256, 0, st>>>(a, w.flat);
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaMemcpyAsync(host_grad, w.flat, (size_t)o * 4, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(host_grad, w.flat, (size_t)sur_nparams() * 4, cudaMemcpyDeviceToHost, st);
     }
     unsigned int h = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, err, 4, cudaMemcpyDeviceToHost, st);
