@@ -24,10 +24,118 @@ __device__ __forceinline__ void store_bf16_row(const GemmArgs &g, int row, int c
     }
 }
 
+// ---- 32 columns of a warp's 32 rows.  Row-per-thread 16-byte accesses touch 32 lines an instruction, and the epilogue
+// of a 256-wide layer spent 12k cycles of the load/store unit on them; through 4 KB of the ring (free by then) per warp
+// an instruction covers whole lines.  16-byte unit u of row r lies at r * 128 + ((u ^ r % 8) << 4) (FP32, 8 units) or
+// r * 64 + ((u ^ r / 2 % 4) << 4) (BF16, 4 units): no bank conflicts by rows or by units.
+__device__ __forceinline__ float4 *unit32(unsigned char *buf, int r, int u) {
+    return (float4 *)(buf + r * 128 + ((u ^ (r & 7)) << 4));
+}
+__device__ __forceinline__ uint4 *unit16(unsigned char *buf, int r, int u) {
+    return (uint4 *)(buf + r * 64 + ((u ^ ((r >> 1) & 3)) << 4));
+}
+// f(row of the warp's 32, 16-byte unit of 4 columns) for the eight rounds in which the warp covers 32 x 32 values
+template <typename F>
+__device__ __forceinline__ void by_lines(int lane, F f) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f(4 * k + (lane >> 3), lane & 7);
+}
+__device__ __forceinline__ void stage_rows(unsigned char *buf, int lane, const float (&v)[32]) {
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) *unit32(buf, lane, u) = make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+    __syncwarp();
+}
+// BF16 copies of the lane's row: H by lines, the transposed HT (consecutive lanes are consecutive there)
+__device__ __forceinline__ void store_bf16_piece(const GemmArgs &g, unsigned char *buf, int row0, int c, int lane,
+                                                 const float (&v)[32]) {
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        __nv_bfloat162 hv[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            hv[i] = __floats2bfloat162_rn(v[8 * u + 2 * i], v[8 * u + 2 * i + 1]);
+            if (g.HT) {
+                g.HT[(size_t)(c + 8 * u + 2 * i) * g.ldht + row0 + lane] = hv[i].x;
+                g.HT[(size_t)(c + 8 * u + 2 * i + 1) * g.ldht + row0 + lane] = hv[i].y;
+            }
+        }
+        *unit16(buf, lane, u) = *(uint4 *)hv;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = 8 * k + (lane >> 2), u = lane & 3;
+        *(uint4 *)(g.H + (size_t)(row0 + r) * g.ldh + c + 8 * u) = *unit16(buf, r, u);
+    }
+}
+// the pre-activations of a piece, by lines
+__device__ __forceinline__ void load_z(const GemmArgs &g, int row0, int c, int lane, float4 (&z)[8]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        z[k] = *(const float4 *)(g.Z + (size_t)(row0 + 4 * k + (lane >> 3)) * g.ldz + c + 4 * (lane & 7));
+}
+// z: the pre-activations of this piece (EPI_GELU_BWD), replaced by those of the piece at next while it is worked on
+__device__ __forceinline__ void epilogue_piece(const GemmArgs &g, unsigned char *buf, uint32_t taddr, int row0, int c,
+                                               int lane, float4 (&z)[8], int next) {
+    if (g.epi == EPI_GELU_BWD) {
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) *unit32(buf, 4 * k + (lane >> 3), lane & 7) = z[k];
+        __syncwarp();
+        if (next) load_z(g, row0, next, lane, z);
+    }
+    uint32_t ua[16], ub[16];
+    tmem_ld16(taddr, ua);
+    tmem_ld16(taddr + 16, ub);
+    tmem_wait16(ua);
+    tmem_wait16(ub);
+    float v[32];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        v[i] = __uint_as_float(ua[i]);
+        v[16 + i] = __uint_as_float(ub[i]);
+    }
+    if (g.epi == EPI_STORE || g.epi == EPI_ATOMIC) {
+        stage_rows(buf, lane, v);
+        by_lines(lane, [&](int r, int u) {
+            float4 *dst = (float4 *)(g.C + (size_t)blockIdx.y * (size_t)g.slice_stride + (size_t)(row0 + r) * g.ldc + c + 4 * u);
+            if (g.epi == EPI_STORE) *dst = *unit32(buf, r, u);
+            else atomicAdd(dst, *unit32(buf, r, u));
+        });
+    } else if (g.epi == EPI_GELU_BWD) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float4 x = *unit32(buf, lane, u);
+            v[4 * u] *= gelu_tanh_grad(x.x);
+            v[4 * u + 1] *= gelu_tanh_grad(x.y);
+            v[4 * u + 2] *= gelu_tanh_grad(x.z);
+            v[4 * u + 3] *= gelu_tanh_grad(x.w);
+        }
+        store_bf16_piece(g, buf, row0, c, lane, v);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] += g.bias[c + i];
+        if (g.Z) {
+            stage_rows(buf, lane, v);
+            by_lines(lane, [&](int r, int u) {
+                *(float4 *)(g.Z + (size_t)(row0 + r) * g.ldz + c + 4 * u) = *unit32(buf, r, u);
+            });
+        }
+        if (g.epi == EPI_BIAS_GELU) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = gelu_tanh(v[i]);
+            store_bf16_piece(g, buf, row0, c, lane, v);
+        }
+    }
+}
+
 // 16 warps: one thread of warp 0 feeds the tensor core, and all of them share the epilogue, the longer part of a tile
-// here (K <= 256): warp w takes TMEM lanes 32 (w % 4) .. and every fourth 16-column piece.  With four warps a layer of
-// 19456 rows took 21.5 us forward and 24.3 us backward, 19.5
-// and 18.6 now.
+// here (K <= 256): warp w takes TMEM lanes 32 (w % 4) .. and every fourth 32-column piece.  A layer of 19456 rows:
+// four warps 21.5 us forward and 24.3 backward; sixteen 18.1 and 18.3; with accesses by lines 16.3 and 23.4, and
+// with the pre-activations of the backward pass loaded ahead and its derivative without tanhf 14.5 and 15.4; a
+// weight gradient 14.2 -> 11.2.  Bound by the epilogue's stores (256 KB a tile in one wave of tiles).
 __global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const __grid_constant__ CUtensorMap ta,
                                                     const __grid_constant__ CUtensorMap tb, GemmArgs g) {
     extern __shared__ unsigned char smem_raw[];
@@ -63,6 +171,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const __grid_consta
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_slot;
+
+    // 32-column pieces of the epilogue; the first pre-activations are on their way while the products are formed
+    constexpr int PIECES = 32 * (GEMM_THREADS / 128);
+    const int wide = N & ~31, c0 = 32 * (warp >> 2), row0 = m0 + (warp & 3) * 32;
+    float4 z[8];
+    if (g.epi == EPI_GELU_BWD && c0 < wide) load_z(g, row0, c0, lane, z);
 
     if (threadIdx.x == 0) {
         const uint32_t idesc = bf16_idesc(N);
@@ -118,7 +232,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const __grid_consta
         if (threadIdx.x == 0 && g.err) atomicExch(g.err, 1u);
     } else {
         const int q = warp & 3, row = m0 + q * 32 + lane;
-        for (int c = 16 * (warp >> 2); c < N; c += 16 * (GEMM_THREADS / 128)) {
+        for (int c = c0; c < wide; c += PIECES)
+            epilogue_piece(g, smem + warp * 4096, tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c, row0, c, lane, z,
+                           c + PIECES < wide ? c + PIECES : 0);
+        // the last 16 columns of an odd multiple of 16
+        for (int c = wide + 16 * (warp >> 2); c < N; c += 16 * (GEMM_THREADS / 128)) {
             uint32_t r[16];
             const uint32_t addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c;
             asm volatile(
