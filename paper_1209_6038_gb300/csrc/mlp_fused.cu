@@ -32,7 +32,8 @@
 // its outputs go straight to the caller's rows: packing to 128-byte rows and unpacking from 64-byte ones moved 340
 // bytes a row in two more launches, and the copy warp's wait for a free tile held up the weights behind it.
 // 1,000,003 rows 605 -> 457 us, bit for bit the same.  Bound now by the
-// epilogue and its hand-over to the MMAs: tensor pipe about a third busy.
+// epilogue (issue slots 68 % busy, tensor pipe 40 %): no weight loads at all, or accumulators released before the
+// GELU, take as long, and 24 epilogue warps longer (485 us).
 // Barriers: full/empty per ring slot; per tile the inputs' barrier, "MMAs done" (committed by the MMA
 // warp), "activations free" (its last layer's) and "activations ready" (16 arrivals).  Shared memory: activations 2 x 64 KB, weight ring
 // 3 x 32 KB.  Every mbarrier wait is bounded; on a timeout the kernel sets the error flag, lets its MMAs and
