@@ -120,69 +120,71 @@ __global__ void k_sur_loss(const float *Y, const float *Tb, int B, int stage, __
     if ((threadIdx.x & 31) == 0 && L != 0.0) atomicAdd(loss, L);
 }
 
-// Gradients of one layer from what its GEMM left, in one launch.
+// Gradients of one layer from what its GEMM left, in one launch.  Both sums are formed in one fixed order, whatever
+// the launch looks like, so that training from a seed always gives the same network; the loads, whose latency bounds
+// this, are not bound to that order: a block brings RED_BYTES into shared memory, all loads of a thread in flight at
+// once, and adds from there.  76 slices of a 256 x 256 layer and its bias 9.5 us (8.4 when eight threads per output
+// added a run of slices each; 11.0 and 38 with one load after the other); a gradient of 19456 rows 311 us.
 // Blocks below wblocks: gW[i] = sum over the slices of part[s * stride + i], i < n (multiples of 4), the batch-split weight
-// gradient, summed the same way on every run (atomic accumulation made training order-dependent): four outputs per
-// load, eight threads per output take a run of slices each and are added in order.  Bound by the latency of a
-// thread's loads: 76 slices of 256 x 256 took 9.0 us with one thread per output and 4.6 more for the bias, both 8.4 here
-// (11.0 and 38 at first); the output layer sums its 5 rows of 128 only.  A gradient of 19456 rows 390 -> 354 us.
-// The others: gb[r] = sum over the columns of row r of the transposed dZ, sixteen bytes per load (cols is a multiple
-// of 128, so rows are aligned); 19456 columns with one value per load took 38 us, 5 in a launch of its own.
-constexpr int RED_THREADS = 512, RED_PARTS = 8, RED_OUT = 4 * RED_THREADS / RED_PARTS;
+// gradient, one slice after the other (the output layer's 5 rows of 128 only).
+// The others: gb[r] = sum over the columns of row r of the transposed dZ (cols is a multiple of 128, so rows are
+// aligned to 16 bytes): thread t takes the columns t, t + 256, ..., and the threads are added by halving.
+constexpr int RED_THREADS = 512, RED_BYTES = 40960, RED_LOADS = RED_BYTES / 16 / RED_THREADS;  // 16-byte loads per thread
+constexpr int RED_OUT = 128, RED_SLICES = RED_BYTES / (4 * RED_OUT);   // weights per block, slices per round
+constexpr int RED_ADDERS = 256;                                        // threads that add a bias row
 __global__ void __launch_bounds__(RED_THREADS) k_sur_reduce(const float *part, int slices, int n, int stride, float *gW,
                                                             int wblocks, const __nv_bfloat16 *dZT, int cols, float *gb) {
+    __shared__ uint4 buf[RED_BYTES / 16];
+    const int tid = threadIdx.x;
+    uint4 v[RED_LOADS];
+    float s = 0.f;
     if ((int)blockIdx.x < wblocks) {
-        constexpr int PER = RED_THREADS / RED_PARTS;
-        const int o = threadIdx.x % PER, g = threadIdx.x / PER, i = blockIdx.x * RED_OUT + 4 * o;
-        const int run = (slices + RED_PARTS - 1) / RED_PARTS, k1 = min(slices, (g + 1) * run);
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < n) {
-#pragma unroll 10
-            for (int k = g * run; k < k1; ++k) {
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(part + (size_t)k * stride + i));
-                acc.x += v.x;
-                acc.y += v.y;
-                acc.z += v.z;
-                acc.w += v.w;
+        constexpr int PER = RED_OUT / 4;  // threads across the block's weights
+        const int first = blockIdx.x * RED_OUT, i = first + 4 * (tid % PER);
+        for (int k0 = 0; k0 < slices; k0 += RED_SLICES) {
+            const int kn = min(RED_SLICES, slices - k0);
+#pragma unroll
+            for (int j = 0; j < RED_LOADS; ++j) {
+                const int k = tid / PER + j * (RED_THREADS / PER);
+                if (k < kn && i < n) v[j] = __ldg(reinterpret_cast<const uint4 *>(part + (size_t)(k0 + k) * stride + i));
             }
+#pragma unroll
+            for (int j = 0; j < RED_LOADS; ++j) buf[tid + j * RED_THREADS] = v[j];
+            __syncthreads();
+            const float *f = reinterpret_cast<const float *>(buf) + tid;
+            if (tid < RED_OUT)
+                for (int k = 0; k < kn; ++k) s += f[k * RED_OUT];
+            __syncthreads();
         }
-        __shared__ float4 sums[RED_PARTS][PER];
-        sums[g][o] = acc;
-        __syncthreads();
-        if (g == 0 && i < n) {
-            for (int k = 1; k < RED_PARTS; ++k) {
-                const float4 v = sums[k][o];
-                acc.x += v.x;
-                acc.y += v.y;
-                acc.z += v.z;
-                acc.w += v.w;
-            }
-            *reinterpret_cast<float4 *>(gW + i) = acc;
-        }
+        if (tid < RED_OUT && first + tid < n) gW[first + tid] = s;
         return;
     }
     const int r = blockIdx.x - wblocks;
     const uint4 *row = reinterpret_cast<const uint4 *>(dZT + (size_t)r * cols);
-    float s = 0.f;
-    for (int c = threadIdx.x; c < cols / 8; c += RED_THREADS) {
-        const uint4 v = __ldg(row + c);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        float p = 0.f;
+    constexpr int ROUND = RED_BYTES / 2;  // columns per round
+    for (int c0 = 0; c0 < cols; c0 += ROUND) {
+        const int cn = min(ROUND, cols - c0);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w[j]));
-            p += f.x + f.y;
+        for (int j = 0; j < RED_LOADS; ++j) {
+            const int u = tid + j * RED_THREADS;
+            if (u < cn / 8) v[j] = __ldg(row + c0 / 8 + u);
         }
-        s += p;
+#pragma unroll
+        for (int j = 0; j < RED_LOADS; ++j) buf[tid + j * RED_THREADS] = v[j];
+        __syncthreads();
+        const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(buf);
+        if (tid < RED_ADDERS)
+            for (int c = tid; c < cn; c += RED_ADDERS) s += __bfloat162float(h[c]);
+        __syncthreads();
     }
-    __shared__ float part_row[RED_THREADS / 32];
+    __shared__ float part_row[RED_ADDERS / 32];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) part_row[threadIdx.x >> 5] = s;
+    if ((tid & 31) == 0 && tid < RED_ADDERS) part_row[tid >> 5] = s;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        s = threadIdx.x < RED_THREADS / 32 ? part_row[threadIdx.x] : 0.f;
+    if (tid < 32) {
+        s = tid < RED_ADDERS / 32 ? part_row[tid] : 0.f;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) gb[r] = s;
+        if (tid == 0) gb[r] = s;
     }
 }
 

@@ -44,3 +44,9 @@ def test_gradient_keeps_its_roundings(gradient, stage, n):
     relative effect is below sqrt(152) 2^-24 = 7.3e-7.  One changed rounding in some hundred thousand dZ is 1e-5."""
     ref = golden(stage, n).astype(np.float64)
     assert np.linalg.norm(gradient(stage, n) - ref) <= 7.3e-7 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("stage,n", M.CASES)
+def test_gradient_sums_in_its_order(gradient, stage, n):
+    """Slices are added one after the other and bias columns in their fixed tree: the same bits."""
+    assert np.array_equal(gradient(stage, n).view(np.uint32), golden(stage, n).view(np.uint32))
