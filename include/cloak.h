@@ -352,7 +352,9 @@ int cloak_surrogate_forward(cloak_t *h, const float *dev_x, long n, float *dev_y
  * confidence target, mask, two unused), n % 128 == 0.  stage 1 or 2 selects the loss (see train).
  * host_grad (nullable): receives the gradient of the mean loss, flat layout of cloak_surrogate_params.
  * lr > 0 also applies one Adam step (beta 0.9 / 0.999, eps 1e-8) with that learning rate.
- * Synchronises cuda_stream. */
+ * Synchronises cuda_stream.  A call's workspace (some 7 KB per row) is kept for the next batch of the same
+ * size by any handle of the process: at most 1 GiB in all, given back with the last handle that has a surrogate, when
+ * cloak_surrogate_train starts, and when an allocation of the library would fail. */
 int cloak_surrogate_step(cloak_t *h, const float *dev_x, const float *dev_t, long n, int stage, double lr,
                          float *host_grad, void *cuda_stream);
 

@@ -171,7 +171,7 @@ static int wavefront_scratch(cloak *h, long long cap, ck::Queue &q, float4 **sam
             h->scratch_bytes = 0;
             if (e != cudaSuccess) return cuda_fail(e, "cudaFree(scratch)");
         }
-        cudaError_t e = cudaMalloc(&h->scratch, need);
+        cudaError_t e = ck::dev_malloc(&h->scratch, need);
         if (e != cudaSuccess) {
             h->scratch = nullptr;
             cudaGetLastError();
@@ -717,7 +717,7 @@ static int batch_core(cloak_t *h, const cloak_view *views, int nviews, int spp, 
             h->batch_bytes = 0;
             if ((e = cudaHostAlloc(&h->batch_host, tbytes, cudaHostAllocDefault)) != cudaSuccess)
                 return fail(CLOAK_ENOMEM, "pinned view table: %s", cudaGetErrorString(e));
-            if ((e = cudaMalloc(&h->batch_dev, tbytes)) != cudaSuccess) {
+            if ((e = ck::dev_malloc(&h->batch_dev, tbytes)) != cudaSuccess) {
                 cudaFreeHost(h->batch_host);
                 h->batch_host = nullptr;
                 return fail(CLOAK_ENOMEM, "device view table: %s", cudaGetErrorString(e));
@@ -818,7 +818,7 @@ extern "C" int cloak_render_panel(cloak_t *h, int panel, int spp, unsigned long 
         if (h->panel_img) cudaFree(h->panel_img);
         h->panel_img = nullptr;
         h->panel_bytes = 0;
-        cudaError_t e = cudaMalloc(&h->panel_img, 2 * npix * 16);
+        cudaError_t e = ck::dev_malloc(&h->panel_img, 2 * npix * 16);
         if (e != cudaSuccess) {
             h->panel_img = nullptr;
             cudaGetLastError();
@@ -851,7 +851,7 @@ extern "C" int cloak_render_panel(cloak_t *h, int panel, int spp, unsigned long 
             if (h->refl_scratch) cudaFree(h->refl_scratch);
             h->refl_scratch = nullptr;
             h->refl_bytes = 0;
-            cudaError_t e = cudaMalloc(&h->refl_scratch, need);
+            cudaError_t e = ck::dev_malloc(&h->refl_scratch, need);
             if (e != cudaSuccess) {
                 h->refl_scratch = nullptr;
                 cudaGetLastError();

@@ -14,6 +14,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -318,7 +320,7 @@ static bool tmap(CUtensorMap *m, const void *base, long long rows, int cols, int
     return make_tmap_bf16(m, base, (int)rows, cols, box_rows) == CUDA_SUCCESS;
 }
 
-static void drop_grad_ws(SurNet *s);
+static void networks(int change);
 SurNet *sur_create(double R1, double R2, double H, unsigned long long seed, const char **why) {
     SurNet *s = new SurNet();
     memset(s, 0, sizeof(*s));
@@ -333,7 +335,7 @@ SurNet *sur_create(double R1, double R2, double H, unsigned long long seed, cons
         bytes += align256((size_t)d.nout * d.kin * 2) + align256((size_t)d.mw * 2);  // Wh, bh
     }
     bytes += 256;  // error flag
-    cudaError_t e = cudaMalloc(&s->arena, bytes);
+    cudaError_t e = dev_malloc((void **)&s->arena, bytes);
     if (e != cudaSuccess) {
         *why = "cannot allocate the surrogate's parameters";
         delete s;
@@ -398,6 +400,7 @@ SurNet *sur_create(double R1, double R2, double H, unsigned long long seed, cons
         delete s;
         return nullptr;
     }
+    networks(1);
     return s;
 }
 
@@ -405,7 +408,7 @@ void sur_destroy(SurNet *s) {
     if (!s) return;
     if (s->inf_arena) cudaFree(s->inf_arena);
     if (s->arena) cudaFree(s->arena);
-    drop_grad_ws(s);
+    networks(-1);
     delete s;
 }
 
@@ -431,7 +434,7 @@ cudaError_t sur_ensure_inference(SurNet *s, long long rows) {
         s->inf_rows = 0;
     }
     const size_t xb = align256((size_t)rows * 64 * 2), yb = align256((size_t)rows * 16 * 4), eb = align256((size_t)rows);
-    cudaError_t e = cudaMalloc(&s->inf_arena, xb + yb + eb);
+    cudaError_t e = dev_malloc((void **)&s->inf_arena, xb + yb + eb);
     if (e != cudaSuccess) return e;
     char *p = s->inf_arena;
     s->X = (uint16_t *)p; p += xb;
@@ -450,7 +453,8 @@ cudaError_t sur_forward(SurNet *s, long long n, const unsigned int *m_count, cud
 
 // ------------------------------------------------------------------ training workspace
 struct TrainWS {
-    int B;
+    int B, dev;
+    TrainWS *next;  // in the list of kept workspaces
     char *arena;
     size_t bytes;
     float *flat;  // the gradient in the C ABI's layout (k_sur_flat_grad)
@@ -478,7 +482,8 @@ static cudaError_t ws_create(TrainWS &w, int B, cudaStream_t st) {
     const size_t flat = align256((size_t)sur_nparams() * 4);
     const size_t bytes = 2 * x + t + 4 * z + 8 * h + y + x + dyt + 4 * h + 512 + part + flat;
     w.bytes = bytes;
-    cudaError_t e = cudaMalloc(&w.arena, bytes);
+    cudaGetDevice(&w.dev);
+    cudaError_t e = dev_malloc((void **)&w.arena, bytes);
     if (e != cudaSuccess) return e;
     // cleared on the stream that uses it (a cudaMemset on the legacy default stream can still be running
     // when the first kernels of a non-blocking stream start)
@@ -511,28 +516,75 @@ static void ws_destroy(TrainWS &w) {
     if (w.arena) cudaFree(w.arena);
     w.arena = nullptr;
 }
-// The workspace of a batch gradient stays with the network for the next batch of the same size, up to this many
-// bytes (allocating and clearing 130 MB took half of a call's time at the training batch); its padding, cleared
-// when it is made, is never written.
+// Workspaces of finished batch gradients, kept for the next batch of the same size (allocating and clearing 130 MB
+// took half of a call's time at the training batch): up to GRAD_WS_KEEP bytes in all, the most recent first.  Every
+// call has waited for its stream before it hands its workspace back, so any stream may take it; a workspace in use is
+// not in the list.  The padding, cleared when a workspace is made, is never written.  They are given back with the
+// last network, when a training starts, and when an allocation of the library finds the device full (dev_malloc).
 constexpr size_t GRAD_WS_KEEP = (size_t)1 << 30;
-static cudaError_t grad_workspace(SurNet *s, int B, cudaStream_t st, TrainWS **out) {
-    if (s->grad_ws && s->grad_ws->B != B) drop_grad_ws(s);
-    if (!s->grad_ws) {
-        s->grad_ws = new TrainWS();
-        const cudaError_t e = ws_create(*s->grad_ws, B, st);
-        if (e != cudaSuccess) {
-            drop_grad_ws(s);
-            return e;
-        }
+static std::mutex g_ws_mu;
+static TrainWS *g_ws_idle = nullptr;
+static int g_networks = 0;
+static void ws_free(TrainWS *w) {
+    while (w) {
+        TrainWS *next = w->next;
+        ws_destroy(*w);
+        delete w;
+        w = next;
     }
-    *out = s->grad_ws;
-    return cudaSuccess;
 }
-static void drop_grad_ws(SurNet *s) {
-    if (!s->grad_ws) return;
-    ws_destroy(*s->grad_ws);
-    delete s->grad_ws;
-    s->grad_ws = nullptr;
+static TrainWS *ws_take(int B) {
+    int dev = -1;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(g_ws_mu);
+    for (TrainWS **p = &g_ws_idle; *p; p = &(*p)->next)
+        if ((*p)->B == B && (*p)->dev == dev) {
+            TrainWS *w = *p;
+            *p = w->next;
+            w->next = nullptr;
+            return w;
+        }
+    return nullptr;
+}
+static void ws_keep(TrainWS *w) {
+    TrainWS *surplus;
+    {
+        std::lock_guard<std::mutex> lock(g_ws_mu);
+        w->next = g_ws_idle;
+        g_ws_idle = w;
+        size_t total = 0;
+        TrainWS **p = &g_ws_idle;
+        while (*p && (total += (*p)->bytes) <= GRAD_WS_KEEP) p = &(*p)->next;
+        surplus = *p;
+        *p = nullptr;
+    }
+    ws_free(surplus);
+}
+static void ws_release() {
+    TrainWS *all;
+    {
+        std::lock_guard<std::mutex> lock(g_ws_mu);
+        all = g_ws_idle;
+        g_ws_idle = nullptr;
+    }
+    ws_free(all);
+}
+static void networks(int change) {
+    int left;
+    {
+        std::lock_guard<std::mutex> lock(g_ws_mu);
+        left = g_networks += change;
+    }
+    if (left == 0) ws_release();
+}
+cudaError_t dev_malloc(void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();  // reported by the return value, not by the next launch's check
+        ws_release();
+        if ((e = cudaMalloc(p, bytes)) != cudaSuccess) cudaGetLastError();
+    }
+    return e;
 }
 
 // split of the batch dimension for the weight-gradient GEMMs: about one CTA per SM
@@ -781,10 +833,18 @@ int sur_forward_rows(SurNet *s, const float *dev_x, long long n, float *dev_y, c
 // gradients (host, flat layout) of one batch, and optionally one Adam step with learning rate lr
 int sur_batch_grad(SurNet *s, const float *dev_x, const float *dev_t, long long n, int stage, double lr,
                    float *host_grad, cudaStream_t st, std::string &why) {
-    TrainWS *kept = nullptr;
-    cudaError_t e = grad_workspace(s, (int)n, st, &kept);
-    if (e != cudaSuccess) { why = "cannot allocate the training workspace"; return CLOAK_ENOMEM; }
-    TrainWS &w = *kept;
+    TrainWS *ws = ws_take((int)n);
+    cudaError_t e = cudaSuccess;
+    if (!ws) {
+        ws = new (std::nothrow) TrainWS();
+        e = ws ? ws_create(*ws, (int)n, st) : cudaErrorMemoryAllocation;
+        if (e != cudaSuccess) {
+            ws_free(ws);
+            why = "cannot allocate the training workspace";
+            return CLOAK_ENOMEM;
+        }
+    }
+    TrainWS &w = *ws;
     unsigned int *err = s->err;  // this network's own timeout flag
     cudaMemsetAsync(err, 0, 4, st);
     cudaMemsetAsync(w.loss, 0, 8, st);
@@ -819,7 +879,8 @@ int sur_batch_grad(SurNet *s, const float *dev_x, const float *dev_t, long long 
     unsigned int h = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, err, 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess || w.bytes > GRAD_WS_KEEP) drop_grad_ws(s);
+    if (e == cudaSuccess) ws_keep(ws);
+    else ws_free(ws);
     if (e != cudaSuccess) { why = cudaGetErrorString(e); return CLOAK_ECUDA; }
     if (h) { why = "tensor-core GEMM timed out"; return CLOAK_ETIMEOUT; }
     return CLOAK_OK;
@@ -838,10 +899,11 @@ int sur_train(SurNet *s, const Params &p, long long n, unsigned long long seed, 
         why = cudaGetErrorString(e);
         return CLOAK_ECUDA;
     }
+    ws_release();
     // 1. training set: the integrator traces n seeded rays
     const size_t qb = queue_bytes(n), xb = (size_t)n * SUR_XSTRIDE * 4, tb = (size_t)n * SUR_TSTRIDE * 4;
     char *data = nullptr;
-    e = cudaMalloc(&data, qb + xb + tb);
+    e = dev_malloc((void **)&data, qb + xb + tb);
     if (e != cudaSuccess) {
         cudaStreamDestroy(st);
         why = "cannot allocate the training set";

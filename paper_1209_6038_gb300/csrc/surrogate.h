@@ -52,7 +52,6 @@ __host__ __device__ inline SurDims sur_dims(int l) {
     return d;
 }
 
-struct TrainWS;
 struct SurNet {
     // parameters, FP32 master copies (W: mw x kin, zero outside out x in; b: mw)
     float *W[SUR_L], *b[SUR_L];
@@ -81,10 +80,11 @@ struct SurNet {
     int inf_f16;  // inference operands: 0 = BF16 (the training precision, default), 1 = FP16
     float *Y;
     unsigned char *elig;
-    // workspace of the last batch gradient, kept for the next of the same size (surrogate.cu)
-    TrainWS *grad_ws;
 };
 
+// cudaMalloc for the library's buffers: on a full device the kept gradient workspaces are given back and it is tried
+// once more; a failure leaves no error behind for the next launch's check (surrogate.cu)
+cudaError_t dev_malloc(void **p, size_t bytes);
 // lifetime and parameters (surrogate.cu)
 SurNet *sur_create(double R1, double R2, double H, unsigned long long seed, const char **why);
 void sur_destroy(SurNet *s);
