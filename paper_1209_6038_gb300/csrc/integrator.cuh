@@ -43,13 +43,14 @@ struct State64 {
     __device__ __forceinline__ double g_end(const Params &p, int ev) const { return event_g(p, ev, y1); }
     __device__ __forceinline__ double g_end_rr(const Params &p, int ev) const { return event_g(p, ev, rr, y1[2]); }
     double rr;  // r^2 at y1, where the step leaves it (DP5(4) of the Fermat form)
-    // surfaces behind the end point: bit ev is set iff event_g(ev, y1) > 0, decided by integer comparisons
+    // surfaces behind the end point: bit ev is set iff event_g(ev, y1) > 0, decided by integer comparisons; none is
+    // where the end point is NaN (a fixed RK4 step that lands on r = R1 exactly: no step control rejects it)
     template <bool RR>
     __device__ __forceinline__ unsigned int crossed_rr(const Params &p, int nev) const {
         const double r2 = RR ? rr : fma(y1[0], y1[0], __dmul_rn(y1[1], y1[1])), az = s64_abs(y1[2]);
         unsigned int m = 0;
-        if (s64_gt_pos(r2, p.R2sq) && !s64_isnan(r2)) m |= 1u << EV_LAT;
-        if (s64_gt_pos(az, p.halfH) && !s64_isnan(az)) m |= __double2hiint(y1[2]) < 0 ? 1u << EV_BOT : 1u << EV_TOP;
+        if (s64_gt_pos(r2, p.R2sq)) m |= 1u << EV_LAT;
+        if (s64_gt_pos(az, p.halfH)) m |= __double2hiint(y1[2]) < 0 ? 1u << EV_BOT : 1u << EV_TOP;
         if (nev == 4 && s64_gt_pos(p.R1sq, r2)) m |= 1u << EV_METAL;
         return m;
     }
@@ -299,11 +300,14 @@ struct StepperWide : State64<INTEG> {
     // dp_control, a component per lane
     __device__ __forceinline__ bool control(double tol, double &fac) const {
         const double sc = fma(tol, fmax(s64_abs(yo), s64_abs(y1o)), tol), ae = s64_abs(eo);
-        const bool bad = s64_isnan(ae);
-        bool ok = true;
+        bool ok = true, bad = false, le = s64_bits(ae) <= s64_bits(sc);
         float fe = __fdividef(s64_to_float(ae, ok), s64_to_float(sc, ok));
-        if (!ok) fe = __fdividef((float)ae, (float)sc);
-        const bool acc = __all_sync(grp, bad || s64_le_pos(ae, sc));
+        if (!ok) {
+            bad = ae != ae;
+            le = ae <= sc;
+            fe = __fdividef((float)ae, (float)sc);
+        }
+        const bool acc = __all_sync(grp, le);
         if (__any_sync(grp, bad)) { fac = 0.2; return false; }
         fe = fmaxf(fe, 0.f);  // NaN (infinite over infinite) counts for nothing, as in dp_control
 #pragma unroll
@@ -852,8 +856,10 @@ __device__ __forceinline__ bool inside(double a, double lo, double hi) {
 __device__ __forceinline__ bool inside(float a, float lo, float hi) { return a > lo && a < hi; }
 __device__ __forceinline__ bool positive(double a) { return s64_positive(a); }
 __device__ __forceinline__ bool positive(float a) { return a > 0.f; }
-__device__ __forceinline__ bool le_pos(double a, double b) { return s64_le_pos(a, b); }  // 0 <= a or NaN, 0 <= b
+__device__ __forceinline__ bool le_pos(double a, double b) { return s64_le_pos(a, b); }  // 0 <= a, b, or NaN
 __device__ __forceinline__ bool le_pos(float a, float b) { return a <= b; }
+__device__ __forceinline__ bool gt_pos(double a, double b) { return s64_gt_pos(a, b); }  // 0 <= a, b, or NaN
+__device__ __forceinline__ bool gt_pos(float a, float b) { return a > b; }
 __device__ __forceinline__ bool not_positive(double a) { return s64_not_positive(a); }
 __device__ __forceinline__ bool not_positive(float a) { return a <= 0.f; }
 __device__ __forceinline__ bool not_negative(double a) { return s64_not_negative(a); }
@@ -910,7 +916,7 @@ struct Lane {
         const R tol = (R)p.h_or_tol;
         const float conv = sizeof(R) == 8 ? (float)CROSS_REL_TOL : 2.4e-7f;  // bracket resolution of the search
         int status = -1;
-        if (phase == PH_STEP && (steps >= p.max_steps || (INTEG == I_DP45 && !le_pos((R)1e-14, h))))
+        if (phase == PH_STEP && (steps >= p.max_steps || (INTEG == I_DP45 && gt_pos((R)1e-14, h))))
             status = CLOAK_RAY_STEP_LIMIT;
         R s = phase == PH_STEP ? h : sbest;
         if (phase == PH_CROSS) {

@@ -597,21 +597,26 @@ __device__ __forceinline__ double dp_factor(float fe) {
 }
 __device__ __forceinline__ bool dp_control(const double y[6], const double y1[6], const double e6[6], double tol,
                                            double &fac) {
-    bool acc = true, bad = false, ok = true;
+    bool acc = true, ok = true;
     float fe = 0.f;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {  // comparisons and conversions on the integer pipes
         const double sc = fma(tol, fmax(s64_abs(y[i]), s64_abs(y1[i])), tol), ae = s64_abs(e6[i]);
-        if (s64_isnan(ae)) bad = true;
-        if (!s64_le_pos(ae, sc)) acc = false;
+        if (s64_bits(ae) > s64_bits(sc)) acc = false;
         fe = fmaxf(fe, __fdividef(s64_to_float(ae, ok), s64_to_float(sc, ok)));
     }
-    if (bad) { fac = 0.2; return false; }
-    if (!ok) {  // an error or scale beyond the float range
+    if (!ok) {  // an error or scale beyond the float range, infinite or NaN
+        bool bad = false;
+        acc = true;
         fe = 0.f;
 #pragma unroll
-        for (int i = 0; i < 6; ++i)
-            fe = fmaxf(fe, __fdividef((float)fabs(e6[i]), (float)fma(tol, fmax(fabs(y[i]), fabs(y1[i])), tol)));
+        for (int i = 0; i < 6; ++i) {
+            const double sc = fma(tol, fmax(fabs(y[i]), fabs(y1[i])), tol), ae = fabs(e6[i]);
+            if (ae != ae) bad = true;
+            if (!(ae <= sc)) acc = false;
+            fe = fmaxf(fe, __fdividef((float)ae, (float)sc));
+        }
+        if (bad) { fac = 0.2; return false; }
     }
     fac = dp_factor(fe);
     return acc;

@@ -132,9 +132,14 @@ S64_FN double s64_half(double a) {
     return s64_make((uint32_t)s64_hi(a) - 0x100000u, (uint32_t)s64_lo(a));
 }
 
-// a <= b and a > b for a, b >= 0 (or +NaN, which orders above infinity), without the FP64 unit
-S64_FN bool s64_le_pos(double a, double b) { return s64_bits(a) <= s64_bits(b); }
-S64_FN bool s64_gt_pos(double a, double b) { return s64_bits(a) > s64_bits(b); }
+// a <= b and a > b without the FP64 unit, for a, b >= 0 (not -0) or NaN of either sign: as the hardware's, false with
+// a NaN (whose bits order above infinity, or below every number)
+S64_FN bool s64_le_pos(double a, double b) {
+    return s64_bits(a) <= s64_bits(b) && s64_bits(a) >= 0 && s64_bits(b) <= 0x7ff0000000000000ll;
+}
+S64_FN bool s64_gt_pos(double a, double b) {
+    return s64_bits(a) > s64_bits(b) && s64_bits(b) >= 0 && s64_bits(a) <= 0x7ff0000000000000ll;
+}
 // a > 0 for any a (false for NaN)
 S64_FN bool s64_positive(double a) {
     const int64_t b = s64_bits(a);
