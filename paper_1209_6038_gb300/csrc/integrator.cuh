@@ -1037,6 +1037,8 @@ struct Lane {
                     newton = false;  // the coarse step's end point is gone: bisection for further surfaces
                     const int e = __ffs(pending) - 1;
                     search(p, st, e == 0 ? g1[0] : e == 1 ? g1[1] : e == 2 ? g1[2] : g1[3]);
+                } else if (!positive(sbest)) {
+                    land = true;  // the step starts on the surface, or behind it by rounding: no trial point before it
                 } else if (S::FP64 && same(sbest, s) && evbest == ev) {
                     land = true;  // the last trial step ended on the crossing: no re-evaluation
                 } else {
@@ -1047,7 +1049,7 @@ struct Lane {
             land = true;  // PH_FINAL: the evaluation landed on the crossing
         }
         if (land) {
-            st.take_crossing();
+            if (positive(sbest)) st.take_crossing();  // else the state at the step's start, which is still there
             t += sbest;
             h = hs * fac;
             phase = PH_STEP;

@@ -484,7 +484,8 @@ static __constant__ double c_dp_e[5] = {DP::e1, DP::e3, DP::e4, DP::e5, DP::e6};
 // Step of size h from y; k1 in slot 0, or evaluated here (first; uniform over the warp: evaluating the k1 that a
 // lane has already gives the same value).  rr: r^2 at y1; y1: the fifth-order solution, e6: the error estimate,
 // slot 6: k7 = f(y1).  h: normal, far from the ends of the exponent range (h >= 1e-14 for a step; a trial
-// size of the crossing search is at least 2^-215 of one).
+// size of the crossing search is at least 2^-215 of one, and a search that ends at the step's start does not
+// evaluate there).
 template <int VAR, int MODE>
 __device__ __forceinline__ void dp45_fermat(const Params &p, const double y[6], double h, bool first, double *kb,
                                             int ks, double y1[6], double e6[6], double &rr) {
