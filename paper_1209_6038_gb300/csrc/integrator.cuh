@@ -866,8 +866,13 @@ __device__ __forceinline__ bool not_negative(double a) { return s64_not_negative
 __device__ __forceinline__ bool not_negative(float a) { return a >= 0.f; }
 __device__ __forceinline__ bool same(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
 __device__ __forceinline__ bool same(float a, float b) { return a == b; }
-// a <= f b for sizes a, b >= 0 whose ratio is decided to single precision
-__device__ __forceinline__ bool below(double a, float f, double b) { return s64_truncate(a) <= f * s64_truncate(b); }
+// a <= f b for sizes 0 <= a <= b whose ratio is decided to single precision: both divided by b's power of two, so that
+// lengths of any scale compare alike
+__device__ __forceinline__ bool below(double a, float f, double b) {
+    const int e = (s64_hi(b) & 0x7ff00000) - 0x3ff00000;
+    const double am = s64_make((uint32_t)max(s64_hi(a) - e, 0), (uint32_t)s64_lo(a));
+    return s64_truncate(am) <= f * s64_truncate(s64_make((uint32_t)(s64_hi(b) - e), (uint32_t)s64_lo(b)));
+}
 __device__ __forceinline__ bool below(float a, float f, float b) { return a <= f * b; }
 __device__ __forceinline__ double mag(double a) { return s64_abs(a); }
 __device__ __forceinline__ float mag(float a) { return fabsf(a); }
