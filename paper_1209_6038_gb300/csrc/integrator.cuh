@@ -968,7 +968,7 @@ struct Lane {
                         for (int e = 0; e < 4; ++e) g1[e] = st.g_end(p, e);
                     }
                     hs = h;
-                    sbest = (R)1e30;
+                    sbest = (R)(S::FP64 ? 1e300 : 1e30);  // above any step
                     evbest = -1;
                     newton = false;
                     fin = false;

@@ -25,7 +25,7 @@ def trace(ck, variant, pol, rays, scale):
 
 @pytest.mark.parametrize("variant,pol", [(0, 0), (0, 1), (1, 0), (1, 1)])
 @pytest.mark.parametrize("rays", [61, 5003])
-@pytest.mark.parametrize("power", [-90, -140, -300])
+@pytest.mark.parametrize("power", [110, 300, -90, -140, -300])
 def test_traces_scale_with_the_geometry(ck, variant, pol, rays, power):
     """Eight lanes per ray and one thread per ray; scales on both sides of the integer products' range (2^-127 .. 2^128)
     and of single precision."""
