@@ -351,11 +351,11 @@ struct StepperHam : State64<INTEG> {
     }
     __device__ __forceinline__ void eval(const Params &p, double s, unsigned int) {
         if (INTEG == I_RK4) {
-            rk4_step<VAR, MODE, true>(p, y, s, y1, vm);
+            rk4_step<VAR, MODE>(p, y, s, y1, vm);
         } else {
             if (need_k1) rhs_ham<VAR, MODE>(p, y, k1, vm);
             need_k1 = false;
-            dp45_step<VAR, MODE, true>(p, y, k1, s, y1, e6, k7, vm);
+            dp45_step<VAR, MODE>(p, y, k1, s, y1, e6, k7, vm);
         }
     }
     __device__ __forceinline__ double g_rate(int ev) const { return event_dg(ev, y1, k7); }
@@ -960,7 +960,7 @@ struct Lane {
                     t += h;
                     h *= fac;
                 } else {
-                                        // the values at the end point, of the further surfaces only if there are any
+                    // the values at the end point, of the further surfaces only if there are any
                     ghi = st.g_end(p, __ffs(pending) - 1);
                     g1[0] = ghi;
                     if (pending & (pending - 1)) {

@@ -97,12 +97,11 @@ __device__ __forceinline__ void epilogue_piece(const GemmArgs &g, unsigned char 
         v[i] = __uint_as_float(ua[i]);
         v[16 + i] = __uint_as_float(ub[i]);
     }
-    if (g.epi == EPI_STORE || g.epi == EPI_ATOMIC) {
+    if (g.epi == EPI_STORE) {
         stage_rows(buf, lane, v);
         by_lines(lane, [&](int r, int u) {
             float4 *dst = (float4 *)(g.C + (size_t)blockIdx.y * (size_t)g.slice_stride + (size_t)(row0 + r) * g.ldc + c + 4 * u);
-            if (g.epi == EPI_STORE) *dst = *unit32(buf, r, u);
-            else atomicAdd(dst, *unit32(buf, r, u));
+            *dst = *unit32(buf, r, u);
         });
     } else if (g.epi == EPI_GELU_BWD) {
 #pragma unroll
@@ -249,14 +248,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const __grid_consta
 #pragma unroll
             for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
             if (row < g.M) {
-                if (g.epi == EPI_STORE || g.epi == EPI_ATOMIC) {
+                if (g.epi == EPI_STORE) {
                     float4 *dst = (float4 *)(g.C + (size_t)blockIdx.y * (size_t)g.slice_stride + (size_t)row * g.ldc + c);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float4 q = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                        if (g.epi == EPI_STORE) dst[i] = q;
-                        else atomicAdd(dst + i, q);
-                    }
+                    for (int i = 0; i < 4; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
                 } else if (g.epi == EPI_GELU_BWD) {
                     const float4 *zi = (const float4 *)(g.Z + (size_t)row * g.ldz + c);
 #pragma unroll

@@ -4,12 +4,11 @@
 //
 // One CTA (16 warps) computes a 128 x N tile (N <= 256, multiple of 16) over one slice of K (split-K:
 // gridDim.y slices).  K is consumed in chunks of 64 elements (128 bytes, one 128B-swizzle row): warp 0 /
-// lane 0 issues the TMA loads of A and B chunks into a 3-stage shared-memory ring and the tcgen05.mma
+// lane 0 issues the TMA loads of A and B chunks into a 2-stage shared-memory ring and the tcgen05.mma
 // instructions (M = 128, K = 16 each, accumulator in tensor memory), committing each stage back to its
 // "empty" barrier.  After the last MMA completes, every warp reads its share of the accumulators with
 // tcgen05.ld and applies the epilogue (row r, column c, accumulator a):
 //   EPI_STORE     C[r, c] = a
-//   EPI_ATOMIC    C[r, c] += a                                (split-K partial sums, FP32 atomics)
 //   EPI_BIAS      Z[r, c] = a + bias[c]
 //   EPI_BIAS_GELU z = a + bias[c]; Z[r, c] = z (if Z); H[r, c] = GELU(z) (BF16); HT[c, r] = H[r, c] (if HT)
 //   EPI_GELU_BWD  g = a * GELU'(Z[r, c]); H[r, c] = g (BF16); HT[c, r] = g (if HT)
@@ -26,14 +25,14 @@
 
 namespace ck {
 
-enum { EPI_STORE = 0, EPI_BIAS_GELU = 1, EPI_BIAS = 2, EPI_ATOMIC = 3, EPI_GELU_BWD = 4 };
+enum { EPI_STORE = 0, EPI_BIAS_GELU = 1, EPI_BIAS = 2, EPI_GELU_BWD = 3 };
 
 struct GemmArgs {
     int M, N, K;                 // M % 128 == 0, N % 16 == 0 (16..256), K % (64 * ksplit) == 0
     int ksplit;                  // slices of K (gridDim.y)
     const unsigned int *m_count; // optional device row count
     long long m_base;            // row of this GEMM's row 0 in the count's numbering (chunked inference)
-    float *C;                    // EPI_STORE / EPI_ATOMIC: C[M x ldc]
+    float *C;                    // EPI_STORE: C[M x ldc]
     int ldc;
     const float *bias;           // [N]
     float *Z;                    // EPI_BIAS*: output (optional for GELU); EPI_GELU_BWD: input

@@ -358,38 +358,20 @@ __device__ __forceinline__ void rhs(const Params &p, const double y[6], double d
 }
 
 // ------------------------------------------------------------------ integrators
-// Steps with the stages in registers: of the Hamiltonian form (HAM), or of the Fermat form with hardware products
-// (the mixed precision's band steps).
-template <int VAR, int MODE, bool HAM>
-__device__ __forceinline__ void rhs_inline(const Params &p, const double y[6], double dy[6], int vm) {
-    if (HAM) {
-        rhs_ham<VAR, MODE>(p, y, dy, vm);
-        return;
-    }
-    dy[0] = y[3]; dy[1] = y[4]; dy[2] = y[5];
-    dy[3] = dy[4] = dy[5] = 0.0;
-    double r2;
-    const int m = VAR != V_ANY ? 2 * VAR + MODE : vm;
-    if (VAR != V_TEST && m == 1)
-        accel64_form<MulHW, V_RADIAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2);
-    else if (VAR != V_TEST && m == 2)
-        accel64_form<MulHW, V_AZIMUTHAL, M_ORD>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2);
-    else if (VAR != V_TEST && m == 3)
-        accel64_form<MulHW, V_AZIMUTHAL, M_EXT>(p.R1, y[0], y[1], y[3], y[4], y[5], dy[3], dy[4], dy[5], r2);
-}
-template <int VAR, int MODE, bool HAM>
+// Steps of the Hamiltonian form, the stages in registers.
+template <int VAR, int MODE>
 __device__ __forceinline__ void rk4_step(const Params &p, const double y[6], double h, double out[6], int vm = 0) {
     double k[6], acc[6], t[6];
-    rhs_inline<VAR, MODE, HAM>(p, y, k, vm);
+    rhs_ham<VAR, MODE>(p, y, k, vm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) { acc[i] = k[i]; t[i] = fma(0.5 * h, k[i], y[i]); }
-    rhs_inline<VAR, MODE, HAM>(p, t, k, vm);
+    rhs_ham<VAR, MODE>(p, t, k, vm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) { acc[i] = fma(2.0, k[i], acc[i]); t[i] = fma(0.5 * h, k[i], y[i]); }
-    rhs_inline<VAR, MODE, HAM>(p, t, k, vm);
+    rhs_ham<VAR, MODE>(p, t, k, vm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) { acc[i] = fma(2.0, k[i], acc[i]); t[i] = fma(h, k[i], y[i]); }
-    rhs_inline<VAR, MODE, HAM>(p, t, k, vm);
+    rhs_ham<VAR, MODE>(p, t, k, vm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) out[i] = fma(h * (1.0 / 6.0), acc[i] + k[i], y[i]);
 }
@@ -410,11 +392,11 @@ struct DP {
                             e6 = 11.0 / 84 - 187.0 / 2100, e7 = -1.0 / 40;
 };
 
-// Fifth-order solution of one DP step of size h from y with first stage k1 = f(y).
-// If err != nullptr also returns k7 = f(out) and the embedded error estimate.
-template <int VAR, int MODE, bool HAM>
+// Fifth-order solution of one DP step of size h from y with first stage k1 = f(y); k7 = f(out) and the embedded error
+// estimate.
+template <int VAR, int MODE>
 __device__ __forceinline__ void dp45_step(const Params &p, const double y[6], const double k1[6], double h,
-                                          double out[6], double *err, double *k7, int vm = 0) {
+                                          double out[6], double err[6], double k7[6], int vm = 0) {
     // stage points y + sum_l (h a_jl) k_l as FMA chains on the scaled coefficients (one FMA per term)
     double k2[6], k3[6], k4[6], k5[6], k6[6], t[6];
     {
@@ -422,46 +404,43 @@ __device__ __forceinline__ void dp45_step(const Params &p, const double y[6], co
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = fma(c1, k1[i], y[i]);
     }
-    rhs_inline<VAR, MODE, HAM>(p, t, k2, vm);
+    rhs_ham<VAR, MODE>(p, t, k2, vm);
     {
         const double c1 = h * DP::a31, c2 = h * DP::a32;
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = fma(c2, k2[i], fma(c1, k1[i], y[i]));
     }
-    rhs_inline<VAR, MODE, HAM>(p, t, k3, vm);
+    rhs_ham<VAR, MODE>(p, t, k3, vm);
     {
         const double c1 = h * DP::a41, c2 = h * DP::a42, c3 = h * DP::a43;
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = fma(c3, k3[i], fma(c2, k2[i], fma(c1, k1[i], y[i])));
     }
-    rhs_inline<VAR, MODE, HAM>(p, t, k4, vm);
+    rhs_ham<VAR, MODE>(p, t, k4, vm);
     {
         const double c1 = h * DP::a51, c2 = h * DP::a52, c3 = h * DP::a53, c4 = h * DP::a54;
 #pragma unroll
         for (int i = 0; i < 6; ++i) t[i] = fma(c4, k4[i], fma(c3, k3[i], fma(c2, k2[i], fma(c1, k1[i], y[i]))));
     }
-    rhs_inline<VAR, MODE, HAM>(p, t, k5, vm);
+    rhs_ham<VAR, MODE>(p, t, k5, vm);
     {
         const double c1 = h * DP::a61, c2 = h * DP::a62, c3 = h * DP::a63, c4 = h * DP::a64, c5 = h * DP::a65;
 #pragma unroll
         for (int i = 0; i < 6; ++i)
             t[i] = fma(c5, k5[i], fma(c4, k4[i], fma(c3, k3[i], fma(c2, k2[i], fma(c1, k1[i], y[i])))));
     }
-    rhs_inline<VAR, MODE, HAM>(p, t, k6, vm);
+    rhs_ham<VAR, MODE>(p, t, k6, vm);
     {
         const double c1 = h * DP::b1, c3 = h * DP::b3, c4 = h * DP::b4, c5 = h * DP::b5, c6 = h * DP::b6;
 #pragma unroll
         for (int i = 0; i < 6; ++i)
             out[i] = fma(c6, k6[i], fma(c5, k5[i], fma(c4, k4[i], fma(c3, k3[i], fma(c1, k1[i], y[i])))));
     }
-    if (err) {
-        rhs_inline<VAR, MODE, HAM>(p, out, k7, vm);
-        const double c1 = h * DP::e1, c3 = h * DP::e3, c4 = h * DP::e4, c5 = h * DP::e5, c6 = h * DP::e6,
-                     c7 = h * DP::e7;
+    rhs_ham<VAR, MODE>(p, out, k7, vm);
+    const double c1 = h * DP::e1, c3 = h * DP::e3, c4 = h * DP::e4, c5 = h * DP::e5, c6 = h * DP::e6, c7 = h * DP::e7;
 #pragma unroll
-        for (int i = 0; i < 6; ++i)
-            err[i] = fma(c7, k7[i], fma(c6, k6[i], fma(c5, k5[i], fma(c4, k4[i], fma(c3, k3[i], c1 * k1[i])))));
-    }
+    for (int i = 0; i < 6; ++i)
+        err[i] = fma(c7, k7[i], fma(c6, k6[i], fma(c5, k5[i], fma(c4, k4[i], fma(c3, k3[i], c1 * k1[i])))));
 }
 
 // ------------------------------------------------------------------ the Fermat form's steps, compact
