@@ -7,10 +7,9 @@
 //     128-byte swizzle) through a 3-slot ring, refilling a slot as soon as the MMAs that read it are done,
 //     and loads each tile's inputs (the K-major layout the MMA reads) once the tile's previous last-layer
 //     MMAs are done -- after the weight chunk of the tile's first job, so that chunk is already on its way;
-//   * the MMA warp (the whole warp in step, one elected lane issuing) issues, per chunk, the four tcgen05.mma (M = 128, K = 16) of the job's tile
-//     (one for the first layer, whose 14 input columns fit one K step) into its TMEM columns (tile t:
-//     256 t .. 256 t + 255) and frees the slot by a commit.  Before a job's
-//     first MMA it waits only for the epilogue of the same tile's previous layer, so the MMAs of one tile
+//   * the MMA warp (the whole warp in step, one elected lane issuing) issues, per chunk, the four tcgen05.mma
+//     (M = 128, K = 16) of the job's tile (one for the first layer, whose 14 input columns fit one K step) into
+//     its TMEM columns (tile t: 256 t .. 256 t + 255) and frees the slot by a commit.  Before a job's first MMA it waits only for the epilogue of the same tile's previous layer, so the MMAs of one tile
 //     run while the epilogue of the other tile runs.  In a branch of one thread the compiler cannot keep the
 //     descriptors and barrier addresses in uniform registers and replays each instruction per active lane: with the
 //     warp in step 1,000,003 rows take 605 us instead of 668 (BF16), and a bare stream of these MMAs with its
@@ -35,8 +34,8 @@
 // epilogue (issue slots 68 % busy, tensor pipe 40 %): no weight loads at all, or accumulators released before the
 // GELU, take as long, and 24 epilogue warps longer (485 us).
 // Barriers: full/empty per ring slot; per tile the inputs' barrier, "MMAs done" (committed by the MMA
-// warp), "activations free" (its last layer's) and "activations ready" (16 arrivals).  Shared memory: activations 2 x 64 KB, weight ring
-// 3 x 32 KB.  Every mbarrier wait is bounded; on a timeout the kernel sets the error flag, lets its MMAs and
+// warp), "activations free" (its last layer's) and "activations ready" (16 arrivals).  Shared memory: activations
+// 2 x 64 KB, weight ring 3 x 32 KB.  Every mbarrier wait is bounded; on a timeout the kernel sets the error flag, lets its MMAs and
 // copies in flight complete, frees TMEM and returns.
 #include "device_once.h"
 #include "sur_physics.cuh"

@@ -132,9 +132,9 @@ __device__ __forceinline__ void epilogue_piece(const GemmArgs &g, unsigned char 
 
 // 16 warps: one thread of warp 0 feeds the tensor core, and all of them share the epilogue, the longer part of a tile
 // here (K <= 256): warp w takes TMEM lanes 32 (w % 4) .. and every fourth 32-column piece.  A layer of 19456 rows:
-// four warps 21.5 us forward and 24.3 backward; sixteen 18.1 and 18.3; with accesses by lines 16.3 and 23.4, and
-// with the pre-activations of the backward pass loaded ahead and its derivative without tanhf 14.5 and 15.4; a
-// weight gradient 14.2 -> 11.2.  Bound by the epilogue's stores (256 KB a tile in one wave of tiles).
+// four warps 21.5 us forward and 24.3 backward; sixteen 18.1 and 18.3; with accesses by lines, and with the
+// pre-activations of the backward pass loaded ahead (23.4 before that), 14.5 and 16.2; a weight gradient 14.2 -> 11.2.
+// Bound by the epilogue's stores (256 KB a tile in one wave of tiles).
 __global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const __grid_constant__ CUtensorMap ta,
                                                     const __grid_constant__ CUtensorMap tb, GemmArgs g) {
     extern __shared__ unsigned char smem_raw[];

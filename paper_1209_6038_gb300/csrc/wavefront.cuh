@@ -323,7 +323,7 @@ __device__ __forceinline__ void wf_integrate_body(const Params &p, const Queue &
     if (VAR == V_ANY) asm("mov.u32 %0, %%smid;" : "=r"(smid));
     int seg = VAR == V_ANY ? 3 - (int)(smid & 3u) : 0;
     // Long-ray blocks: the sort reserved the first rl rays of the order (of medium segment rv in a
-    // batch) -- those that pass closest to the inner radius, up to ~3e4 steps each -- for the warps of
+    // batch) -- those that pass closest to the inner radius, up to 3.4e4 steps each -- for the warps of
     // the first p.dedicated_blocks blocks.  The other blocks resident on those SMs leave at once, so
     // these warps share their SM's FP64 unit with no others and advance their long rays at close to
     // one warp's latency (FP64: four rays per warp, eight lanes each); on a full SM they would get a fraction
