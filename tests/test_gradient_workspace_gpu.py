@@ -106,3 +106,31 @@ def test_kept_memory_is_bounded(ck):
     assert before - free(torch) < 1024 * MB + 64 * MB
     for c in cs:
         c.close()
+
+
+def test_threads_with_handles_of_their_own(ck):
+    """Four threads, each with its handle and stream, take and hand back workspaces of the same sizes at once."""
+    import threading
+    import torch
+    plan = [(1, 2560, 0), (1, 256, 1), (2, 2560, 2), (1, 2560, 3), (1, 256, 4), (1, 2560, 5)]
+    ref = []
+    for stage, n, seed in plan:
+        c = network(ck, M.params())
+        ref.append(step(ck, c, stage, n, seed))
+        c.close()
+    wrong = []
+
+    def work(k):
+        c, s = network(ck, M.params()), torch.cuda.Stream()
+        for i in [(j + k) % len(plan) for j in range(3 * len(plan))]:
+            stage, n, seed = plan[i]
+            if not np.array_equal(step(ck, c, stage, n, seed, 0.0, s), ref[i]):
+                wrong.append((k, i))
+        c.close()
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
