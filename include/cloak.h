@@ -143,7 +143,7 @@ int cloak_set_schedule(cloak_t *h, int schedule, int packet, int steps_per_round
  * records do not depend on them, only the time does): long_ray_blocks (0..64, default 4) blocks of the
  * persistent kernel, each on an SM of its own, take the slowest rays first -- those passing closest to
  * the axis; reserve_per_thread (1..8, default 1) rays are reserved for them per thread (CLOAK_FP64's Fermat form,
- * which advances a ray on eight threads: per eight threads, four times that in a batch); cost_scale
+ * which advances a ray on eight threads: per eight threads, four times that above 2^26 samples); cost_scale
  * (1..16, default 4) sets the resolution of the sort's cost buckets, bucket = cost_scale x -log2 |L_z|
  * (64 buckets).  CLOAK_EINVAL outside these ranges.  Until this call is made on a handle, CLOAK_MIXED and
  * CLOAK_MIXED_FF use their own defaults (16, 4, 3): the slow near-axis rays weigh more in their shorter

@@ -280,7 +280,7 @@ static cudaError_t batch_ip(const Params &p, const ViewDev *views, int nviews, i
     int pk = packet > 0 ? packet : 128;
     // the slowest rays of the batch go to the warps of LONG_RAY_BLOCKS blocks that have their SMs to
     // themselves (k_wf_integrate)
-    k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS_BATCH, long_ray_reserve(p, PREC, pk, true));
+    k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS_BATCH, long_ray_reserve(p, PREC, pk, total));
     k_wf_sort_scatter<<<sms * 8, 256, 0, st>>>(q);
     mark(ev, 1, st);
     Params pl = p;

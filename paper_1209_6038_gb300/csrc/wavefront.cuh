@@ -467,11 +467,13 @@ constexpr auto wf_integrate_kernel() {
     else return k_wf_integrate_mixed<VAR, MODE, INTEG, PREC>;
 }
 // Rays reserved for the long-ray blocks: reserve_per_thread for each of their threads; FP64 Fermat form, where a
-// ray takes eight: reserve_per_thread for each ray that they advance at a time, in a batch four times that
-// (twelve views 1920 x 1080 x 4: one 651, four 622, eight 622 ms; single images, whose bulk is done before the
-// slowest ray: 481 x 271 x 3 one 58.8, four 70.0, eight 96 ms, 1920 x 1080 x 4 one 188, four 209).
-inline unsigned int long_ray_reserve(const Params &p, int prec, int packet, bool batch) {
-    const int per_block = prec == 0 ? (batch ? 4 : 1) * (packet / WIDE_LANES) : packet;
+// ray takes eight: reserve_per_thread for each ray that they advance at a time, four times that in a render of more than
+// 2^26 samples, whose bulk lasts as long as four of the slowest rays one after the other (integration of twelve views of
+// 1920 x 1080 x 4, 99.5 M samples: one 651, four 622, eight 622 ms).  In smaller ones the reserved rays end last, the
+// other SMs idle: twelve views of 1920 x 1080 x 2 one 348, four 350 ms; 960 x 540 x 4 one 183, four 201; 300 x 168 one 13.3,
+// four 25.6; 96 x 54 one 6.0, four 15.7; images 481 x 271 x 3 one 58.8, four 70.0, 1920 x 1080 x 4 one 188, four 209.
+inline unsigned int long_ray_reserve(const Params &p, int prec, int packet, long long samples) {
+    const int per_block = prec == 0 ? (samples > (1LL << 26) ? 4 : 1) * (packet / WIDE_LANES) : packet;
     return (unsigned int)(p.long_ray_blocks * per_block * p.reserve_per_thread);
 }
 // the kernel's precision index from the handle's settings
@@ -573,7 +575,7 @@ static cudaError_t wavefront_vmip(const Params &p, int spp, unsigned long long s
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int pk = packet > 0 ? packet : 128;
     // the slowest rays go to the warps of LONG_RAY_BLOCKS blocks that have their SMs to themselves
-    k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS, long_ray_reserve(p, PREC, pk, false));
+    k_wf_sort_scan<<<1, 32, 0, st>>>(q, NBINS, long_ray_reserve(p, PREC, pk, n));
     k_wf_sort_scatter<<<sms * 8, 256, 0, st>>>(q);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
