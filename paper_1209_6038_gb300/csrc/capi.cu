@@ -100,6 +100,9 @@ static int make_params(const cloak *h, ck::Params &p) {
     p.gtol_lat = ck::CROSS_G_TOL * p.R2sq;
     p.gtol_cap = ck::CROSS_G_TOL * p.halfH;
     p.gtol_metal = ck::CROSS_G_TOL * p.R1sq;
+    p.gtolf_lat = (float)p.gtol_lat;
+    p.gtolf_cap = (float)p.gtol_cap;
+    p.gtolf_metal = (float)p.gtol_metal;
     p.eo_t = h->eo_t;
     p.ee_t = h->ee_t;
     double cl = std::sqrt(h->c_t[0] * h->c_t[0] + h->c_t[1] * h->c_t[1] + h->c_t[2] * h->c_t[2]);

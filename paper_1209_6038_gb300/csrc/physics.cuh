@@ -69,6 +69,7 @@ struct Params {
     float R1f, R2f, halfHf, Kf, invKf, R1sq_hf, R1sq_lf, band_limf;
     float R2sq_hf, R2sq_lf, halfH_hf, halfH_lf;
     double gtol_lat, gtol_cap, gtol_metal;  // |g| at which a point counts as on the surface
+    float gtolf_lat, gtolf_cap, gtolf_metal;  // the same for the mixed steppers (no conversion in their search)
     int dedicated_blocks;  // batched integration: blocks whose warps take the reserved long rays
     // schedule knobs (results do not depend on them): blocks for the slowest rays, rays reserved for them
     // per thread, resolution of the cost buckets (bucket = cost_scale x -log2 |L_z|)
@@ -661,8 +662,11 @@ constexpr double CROSS_REL_TOL = 1e-13;
 // R1^2 or H/2): the point lies on the surface to the rounding of g.
 constexpr double CROSS_G_TOL = 4e-16;
 // (CROSS_G_TOL x R2^2, H/2, H/2, R1^2 for the four surfaces, rounded on the host)
-__device__ __forceinline__ double cross_g_tol(const Params &p, int ev) {
-    return ev == EV_LAT ? p.gtol_lat : ev == EV_METAL ? p.gtol_metal : p.gtol_cap;
+__device__ __forceinline__ void cross_g_tol(const Params &p, int ev, double &tol) {
+    tol = ev == EV_LAT ? p.gtol_lat : ev == EV_METAL ? p.gtol_metal : p.gtol_cap;
+}
+__device__ __forceinline__ void cross_g_tol(const Params &p, int ev, float &tol) {
+    tol = ev == EV_LAT ? p.gtolf_lat : ev == EV_METAL ? p.gtolf_metal : p.gtolf_cap;
 }
 
 // First entry of o + s d into the finite cylinder r <= R2, |z| <= H/2.

@@ -49,6 +49,7 @@ extern "C" int lane_trace(int kind, int vm, double R1, double R2, double H, doub
     p.invK = 1.0 / p.K;
     p.R1x2 = 2 * R1; p.R1sq = R1 * R1; p.R2sq = R2 * R2;
     p.gtol_lat = ck::CROSS_G_TOL * p.R2sq; p.gtol_cap = ck::CROSS_G_TOL * p.halfH; p.gtol_metal = ck::CROSS_G_TOL * p.R1sq;
+    p.gtolf_lat = (float)p.gtol_lat; p.gtolf_cap = (float)p.gtol_cap; p.gtolf_metal = (float)p.gtol_metal;
     p.R1f = (float)R1; p.R2f = (float)R2; p.halfHf = (float)p.halfH; p.Kf = (float)p.K; p.invKf = (float)p.invK;
     p.R1sq_hf = (float)p.R1sq; p.R1sq_lf = (float)(p.R1sq - (double)p.R1sq_hf);
     p.R2sq_hf = (float)p.R2sq; p.R2sq_lf = (float)(p.R2sq - (double)p.R2sq_hf);
