@@ -122,8 +122,9 @@ struct Stepper64 : State64<INTEG> {
         if (INTEG == I_RK4) rk4_fermat<V, M>(p, y, s, y1);
         else dp45_fermat<V, M>(p, y, s, first, kb, ks, y1, e6, rr);
     }
-    // lanes: the lanes of the warp that evaluate with this one
-    __device__ __forceinline__ void eval(const Params &p, double s, unsigned int lanes) {
+    // lanes: the lanes of the warp that evaluate with this one; whole: the error estimate and the derivative at the end
+    // are wanted too (StepperHam on the plain path; the others form them in any case)
+    __device__ __forceinline__ void eval(const Params &p, double s, unsigned int lanes, bool) {
         const bool first = INTEG == I_DP45 && __any_sync(lanes, need_k1);
         if (VAR != V_ANY) {
             eval_medium<VAR, MODE>(p, s, first);
@@ -285,7 +286,7 @@ struct StepperWide : State64<INTEG> {
         }
         need_k1 = false;
     }
-    __device__ __forceinline__ void eval(const Params &p, double h, unsigned int) {
+    __device__ __forceinline__ void eval(const Params &p, double h, unsigned int, bool) {
         if (VAR != V_ANY) {
             eval_medium<VAR, MODE>(p, h);
         } else {
@@ -349,13 +350,13 @@ struct StepperHam : State64<INTEG> {
         y[3] = q.vx[k]; y[4] = q.vy[k]; y[5] = q.vz[k];
         need_k1 = true;
     }
-    __device__ __forceinline__ void eval(const Params &p, double s, unsigned int) {
+    __device__ __forceinline__ void eval(const Params &p, double s, unsigned int, bool whole) {
         if (INTEG == I_RK4) {
             rk4_step<VAR, MODE>(p, y, s, y1, vm);
         } else {
             if (need_k1) rhs_ham<VAR, MODE>(p, y, k1, vm);
             need_k1 = false;
-            dp45_step<VAR, MODE>(p, y, k1, s, y1, e6, k7, vm);
+            dp45_step<VAR, MODE>(p, y, k1, s, y1, whole, e6, k7, vm);
         }
     }
     __device__ __forceinline__ double g_rate(int ev) const { return event_dg(ev, y1, k7); }
@@ -648,7 +649,7 @@ struct StepperMixed {
 #pragma unroll
         for (int i = 2; i < 6; ++i) t[i] = yh[i] + (yl[i] + d[i]);
     }
-    __device__ __forceinline__ void eval(const Params &p, float s, unsigned int) {
+    __device__ __forceinline__ void eval(const Params &p, float s, unsigned int, bool) {
         if (p.band_df && island(p)) {  // double-float step from the float-float state
             df y[6], yo[6], e[6];
 #pragma unroll
@@ -946,7 +947,7 @@ struct Lane {
         const unsigned int on = S::FP64 ? __ballot_sync(lanes, status < 0) : 0u;
         __syncwarp(lanes);  // a convergence point: keeps the compiler from splitting the evaluation by phase
         if (status >= 0) return status;
-        st.eval(p, s, on);
+        st.eval(p, s, on, !EXACT || phase == PH_STEP);
         bool land = false;
         // mixed: the search for the next pending surface starts at one place (gnew: the surface's value at the end point),
         // which keeps a warp's lanes together: images of 128 x 96 and below 1 to 2 % faster; FP64 RK4 rays 3 % slower
