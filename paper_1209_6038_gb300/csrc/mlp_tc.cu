@@ -130,12 +130,13 @@ __device__ __forceinline__ void epilogue_piece(const GemmArgs &g, unsigned char 
     }
 }
 
-// 16 warps: one thread of warp 0 feeds the tensor core, and all of them share the epilogue, the longer part of a tile
-// here (K <= 256): warp w takes TMEM lanes 32 (w % 4) .. and every fourth 32-column piece.  A layer of 19456 rows:
-// four warps 21.5 us forward and 24.3 backward; sixteen 18.1 and 18.3; with accesses by lines, and with the
-// pre-activations of the backward pass loaded ahead (23.4 before that), 14.5 and 16.2; a weight gradient 14.2 -> 11.2.
-// Bound by the epilogue's stores (256 KB a tile in one wave of tiles).
-__global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const __grid_constant__ CUtensorMap ta,
+// THREADS / 32 warps (16 in a network's layers): one thread of warp 0 feeds the tensor core, and all of them share the
+// epilogue, the longer part of a tile here (K <= 256): warp w takes TMEM lanes 32 (w % 4) .. and every THREADS / 128 th
+// 32-column piece.  A layer of 19456 rows: four warps 21.5 us forward and 24.3 backward; sixteen 18.1 and 18.3; with
+// accesses by lines, and with the pre-activations of the backward pass loaded ahead (23.4 before that), 14.5 and 16.2; a
+// weight gradient 14.2 -> 11.2.  Bound by the epilogue's stores (256 KB a tile in one wave of tiles).
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) k_gemm_tc(const __grid_constant__ CUtensorMap ta,
                                                     const __grid_constant__ CUtensorMap tb, GemmArgs g) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[GEMM_STAGES], empty_bar[GEMM_STAGES], done_bar;
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const __grid_consta
     const uint32_t tmem = tmem_slot;
 
     // 32-column pieces of the epilogue; the first pre-activations are on their way while the products are formed
-    constexpr int PIECES = 32 * (GEMM_THREADS / 128);
+    constexpr int PIECES = 32 * (THREADS / 128);
     const int wide = N & ~31, c0 = 32 * (warp >> 2), row0 = m0 + (warp & 3) * 32;
     float4 z[8];
     if (g.epi == EPI_GELU_BWD && c0 < wide) load_z(g, row0, c0, lane, z);
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const __grid_consta
             epilogue_piece(g, smem + warp * 4096, tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c, row0, c, lane, z,
                            c + PIECES < wide ? c + PIECES : 0);
         // the last 16 columns of an odd multiple of 16
-        for (int c = wide + 16 * (warp >> 2); c < N; c += 16 * (GEMM_THREADS / 128)) {
+        for (int c = wide + 16 * (warp >> 2); c < N; c += 16 * (THREADS / 128)) {
             uint32_t r[16];
             const uint32_t addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c;
             asm volatile(
@@ -323,17 +324,20 @@ cudaError_t launch_gemm_tc(const CUtensorMap &ta, const CUtensorMap &tb, const G
     // Shared memory per CTA: the ring, padded so that no more CTAs share an SM than its 512 TMEM columns
     // hold (each allocates the power of two >= N, at least 32) -- an allocation never has to wait.
     static DeviceOnce once;
-    static int smem_sm_of[MAX_DEVICES], reserved_of[MAX_DEVICES], max_dyn_of[MAX_DEVICES];
+    static int smem_sm_of[MAX_DEVICES], reserved_of[MAX_DEVICES], max_dyn_of[MAX_DEVICES], sms_of[MAX_DEVICES];
     cudaError_t e0 = once.run([](int dev) {
         int optin = 0;
         cudaDeviceGetAttribute(&smem_sm_of[dev], cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        cudaDeviceGetAttribute(&sms_of[dev], cudaDevAttrMultiProcessorCount, dev);
         cudaDeviceGetAttribute(&reserved_of[dev], cudaDevAttrReservedSharedMemoryPerBlock, dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, k_gemm_tc);
+        cudaError_t e = cudaFuncGetAttributes(&fa, k_gemm_tc<GEMM_THREADS>);  // static shared memory: the same in both
         if (e != cudaSuccess) return e;
         max_dyn_of[dev] = optin - (int)fa.sharedSizeBytes;  // the barriers are static shared memory
-        return cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn_of[dev]);
+        for (auto kern : {k_gemm_tc<GEMM_THREADS>, k_gemm_tc<128>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn_of[dev]);
+        return e;
     });
     if (e0 != cudaSuccess) return e0;
     int dev = 0;
@@ -346,7 +350,16 @@ cudaError_t launch_gemm_tc(const CUtensorMap &ta, const CUtensorMap &tb, const G
     const size_t floor_b = (size_t)smem_sm / (size_t)(max_ctas + 1) + 1;
     if (smem + (size_t)reserved < floor_b) smem = floor_b - (size_t)reserved;
     if (smem > (size_t)max_dyn) return cudaErrorInvalidValue;
-    k_gemm_tc<<<dim3(g.M / GEMM_TILE_M, g.ksplit), GEMM_THREADS, smem, st>>>(ta, tb, g);
+    const dim3 grid(g.M / GEMM_TILE_M, g.ksplit);
+    // One wave of tiles, or a GELU in the epilogue: 16 warps share each tile's epilogue.  More tiles than SMs with a plain
+    // epilogue: four warps a tile and up to four tiles an SM, whose loads, products and stores overlap (16 warps fill an
+    // SM's registers with one tile).  262144 rows, K = 256, 16 -> 4 warps: N = 16 91.9 -> 53.5 us, 64 102.6 -> 64.1, 256
+    // 139.4 -> 104.9; 19584 rows (153 tiles), N = 16 40.3 -> 32.3; 19456 rows (152), N = 256 39.6 and 40.2.  A gradient
+    // of 131072 rows, GELU layers on 4 warps, 2447 us instead of 2377.
+    if ((long long)grid.x * grid.y > sms_of[dev] && (g.epi == EPI_STORE || g.epi == EPI_BIAS))
+        k_gemm_tc<128><<<grid, 128, smem, st>>>(ta, tb, g);
+    else
+        k_gemm_tc<GEMM_THREADS><<<grid, GEMM_THREADS, smem, st>>>(ta, tb, g);
     return cudaGetLastError();
 }
 

@@ -2,7 +2,7 @@
 //
 //   C[M x N] = A[M x K] * B[N x K]^T      A, B row-major BF16 (K contiguous), FP32 accumulation.
 //
-// One CTA (16 warps) computes a 128 x N tile (N <= 256, multiple of 16) over one slice of K (split-K:
+// One CTA (16 warps, or 4 where there are more tiles than SMs: launch_gemm_tc) computes a 128 x N tile (N <= 256, multiple of 16) over one slice of K (split-K:
 // gridDim.y slices).  K is consumed in chunks of 64 elements (128 bytes, one 128B-swizzle row): warp 0 /
 // lane 0 issues the TMA loads of A and B chunks into a 2-stage shared-memory ring and the tcgen05.mma
 // instructions (M = 128, K = 16 each, accumulator in tensor memory), committing each stage back to its
